@@ -73,7 +73,12 @@ extern "C" {
 #define LBM_COLLIDE_MRT 1 /* Eq. 6: M^-1 S M with S = diag[1, s_e, s_eps, 1, s_q, 1, s_q, 1/tau, 1/tau] */
 
 /* ---- step kernel variants --------------------------------------------- */
-#define LBM_KERNEL_AUTO 0   /* the tuned default for the storage type */
+#define LBM_KERNEL_AUTO 0   /* the library's choice: the storage type's default kernel (which
+                               lbm_get_kernel names); with float storage, no explicit shape and
+                               no CTAs per SM given, two steps at a time run in one pass over
+                               memory, up to 64 per launch (bit-identical; single lattices
+                               with either bounce-back, and batches), and an odd step on the
+                               default kernel */
 #define LBM_KERNEL_DIRECT 1 /* one thread per cell, loads straight from HBM */
 #define LBM_KERNEL_TMA 2    /* persistent; bulk-async (TMA) row staging */
 #define LBM_KERNEL_TMA_BULK 3 /* TMA row staging and TMA bulk stores of the new rows
@@ -286,7 +291,7 @@ int lbm_set_fault_injection(lbm_ctx *ctx, int64_t tile, double wait_seconds);
 int lbm_get_stream(lbm_ctx *ctx, void **stream);
 
 /* Step-kernel launches issued since creation (counts each kernel once; a
- * launch of LBM_KERNEL_TMA_WAVE counts 2, with its force reduction). */
+ * launch of several steps counts 2, with its force reduction). */
 int lbm_launch_count(lbm_ctx *ctx, int64_t *count);
 
 /* Algorithmic bytes one step moves through HBM: 2 * 9 * element size per

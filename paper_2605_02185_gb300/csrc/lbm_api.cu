@@ -15,6 +15,7 @@
 #include "lbm_internal.h"
 #include "lbm_ctx.h"
 #include "lbm_host.h"
+#include "lbm_pair_host.h"
 
 using namespace gblbm;
 
@@ -22,7 +23,7 @@ using namespace gblbm;
 
 namespace {
 
-constexpr int kLayoutParts = 10;
+constexpr int kLayoutParts = 11;
 
 size_t layout(const lbm_opts *o, const Geometry &g, int *pitch_out, size_t offs[kLayoutParts], int *slot_cap_out,
               int *band_rows_out) {
@@ -52,7 +53,8 @@ size_t layout(const lbm_opts *o, const Geometry &g, int *pitch_out, size_t offs[
   offs[6] = off; off += staging;
   offs[7] = off; off += wave_slots;
   offs[8] = off; off += wave_rows;
-  offs[9] = off;
+  offs[9] = off; off += o->storage == LBM_F32 ? pair_region_bytes(kPairCellsSingle, kPairSlotsSingle, 1) : 0;
+  offs[10] = off;
   *pitch_out = pitch;
   *slot_cap_out = slot_cap;
   *band_rows_out = band_rows;
@@ -163,6 +165,38 @@ int configure_kernel(lbm_ctx *c, int kernel, int shape, int ctas_per_sm) {
   return LBM_OK;
 }
 
+// The two-step kernel, for contexts that leave the kernel to the library
+// (LBM_KERNEL_AUTO, no explicit shape).
+int configure_pair(lbm_ctx *c, bool automatic) {
+  c->pair = false;
+  c->pair_auto = automatic;
+  c->pair_grid = 0;
+  if (!automatic || c->o.storage != LBM_F32 || c->kernel != LBM_KERNEL_TMA) return LBM_OK;
+  CK(pair_f32(0, nullptr, nullptr, c->p, c->pq, nullptr, 1, nullptr));
+  int occ = 0;
+  CK(pair_f32(0, nullptr, nullptr, c->p, c->pq, nullptr, 2, &occ));
+  if (occ < 1) return LBM_OK;
+  const int rc = pair_plan({{c->nx, c->ny, c->p.bc, &c->geo}}, c->sms, c->pair_region, kPairCellsSingle, kPairSlotsSingle,
+                           c->stream, &c->pq, &c->pair_grid);
+  if (rc) return rc;
+  c->pq.case_slots = nullptr;
+  c->pair = c->pair_grid > 0;
+  return LBM_OK;
+}
+
+// n steps (even), in passes of two.
+int pair_steps(lbm_ctx *c, int64_t n) {
+  while (n > 0) {
+    PairParams q = c->pq;
+    q.pairs = (int)std::min<int64_t>(n / 2, c->pq.pairs);
+    CK(pair_f32(c->pair_grid, c->buf[c->cur], c->buf[c->cur ^ 1], c->p, q, c->stream, 0, nullptr));
+    c->cur ^= q.pairs & 1;
+    c->launches += 2;
+    n -= 2 * q.pairs;
+  }
+  return LBM_OK;
+}
+
 cudaError_t launch_step(lbm_ctx *c, int from) {
   const void *A = c->buf[from];
   void *B = c->buf[from ^ 1];
@@ -172,10 +206,14 @@ cudaError_t launch_step(lbm_ctx *c, int from) {
   return c->ops->tma(c->shape, c->grid, A, B, c->p, c->stream);
 }
 
-// Clear the multi-step kernel's row counters (a new state, or the recovery
+// Clear the multi-step kernels' counters (a new state, or the recovery
 // from a launch that gave up and left them uneven).
 cudaError_t reset_wave_rows(lbm_ctx *c) {
   c->wave_base = 0;
+  if (c->pair) {
+    const cudaError_t e = pair_reset(c->pq, c->stream);
+    if (e != cudaSuccess) return e;
+  }
   return cudaMemsetAsync(c->wave_rows, 0, (size_t)c->ny * sizeof(unsigned), c->stream);
 }
 
@@ -208,7 +246,7 @@ int capture_graph(lbm_ctx *c) {
     c->graph = nullptr;
   }
   int gs = c->o.graph_steps;
-  if (gs < 0 || c->kernel == LBM_KERNEL_TMA_WAVE) {  // the multi-step kernel needs no graph
+  if (gs < 0 || c->kernel == LBM_KERNEL_TMA_WAVE || c->pair) {  // the multi-step kernels need no graph
     c->graph_steps = 0;
     return LBM_OK;
   }
@@ -318,6 +356,7 @@ int lbm_create_ex(const lbm_opts *o, const uint8_t *mask, lbm_ctx **out) {
   c->staging_bytes = offs[7] - offs[6];
   c->wave_slots = (double2 *)(base + offs[7]);
   c->wave_rows = (unsigned *)(base + offs[8]);
+  c->pair_region = base + offs[9];
   if (o->stream) {
     c->stream = (cudaStream_t)o->stream;
   } else {
@@ -371,6 +410,9 @@ int lbm_create_ex(const lbm_opts *o, const uint8_t *mask, lbm_ctx **out) {
                                    o->cells_per_thread, o->stages, o->ctas_per_sm, &shape, &ctas);
   if (kernel < 0) return fail(LBM_ERR_ARG);
   rc = configure_kernel(c, kernel, std::max(shape, 0), ctas);
+  if (rc) return fail(rc);
+  rc = configure_pair(c, o->kernel == LBM_KERNEL_AUTO && !o->consumer_warps && !o->cells_per_thread && !o->stages &&
+                             o->ctas_per_sm <= 0);
   if (rc) return fail(rc);
   rc = capture_graph(c);
   if (rc) return fail(rc);
@@ -441,6 +483,11 @@ int lbm_step(lbm_ctx *c, int64_t n) {
   if (!c->inited) return LBM_ERR_STATE;
   CK(cudaSetDevice(c->dev));
   if (c->kernel == LBM_KERNEL_TMA_WAVE) return wave_steps(c, n);
+  if (c->pair) {
+    const int rc = pair_steps(c, n & ~(int64_t)1);
+    if (rc) return rc;
+    n &= 1;
+  }
   while (n > 0) {
     if (c->graph && c->cur == 0 && n >= c->graph_steps) {
       CK(cudaGraphLaunch(c->graph, c->stream));
@@ -596,10 +643,13 @@ int lbm_set_kernel(lbm_ctx *c, int kernel, int ncw, int cpt, int stages, int cta
   CK(cudaSetDevice(c->dev));
   CK(cudaStreamSynchronize(c->stream));
   int shape = -1, ctas = 1;
+  const bool automatic = kernel == LBM_KERNEL_AUTO && !ncw && !cpt && !stages && ctas_per_sm <= 0;
   kernel = choose_kernel(c->o.storage, c->nx, c->ny, c->qmap != nullptr, kernel, ncw, cpt, stages, ctas_per_sm, &shape,
                          &ctas);
   if (kernel < 0) return LBM_ERR_ARG;
-  const int rc = configure_kernel(c, kernel, std::max(shape, 0), ctas);
+  int rc = configure_kernel(c, kernel, std::max(shape, 0), ctas);
+  if (rc) return rc;
+  rc = configure_pair(c, automatic);
   if (rc) return rc;
   return capture_graph(c);
 }
@@ -611,6 +661,7 @@ int lbm_set_fault_injection(lbm_ctx *c, int64_t tile, double wait_seconds) {
   if (tile >= (int64_t)c->ny * c->nseg || !(wait_seconds <= 60.0)) return LBM_ERR_ARG;
   CK(cudaSetDevice(c->dev));
   CK(cudaStreamSynchronize(c->stream));
+  c->pair = c->pair_grid > 0 && c->pair_auto && tile < 0 && !(wait_seconds > 0);  // the injection is the one-step kernel's
   c->p.fault_tile = tile < 0 ? -1 : (int)tile;
   c->p.wait_ns = wait_seconds > 0 ? (unsigned long long)(wait_seconds * 1e9) : 1000000000ull;
   if (c->p.wait_ns == 0) c->p.wait_ns = 1;

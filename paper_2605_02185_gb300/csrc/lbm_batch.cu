@@ -19,6 +19,7 @@
 #include "../../include/gblbm.h"
 #include "lbm_ctx.h"
 #include "lbm_host.h"
+#include "lbm_pair_host.h"
 
 using namespace gblbm;
 
@@ -39,6 +40,11 @@ struct lbm_batch {
   long long launches = 0;
   cudaGraphExec_t graph = nullptr;
   int graph_steps = 0;
+  // two-step kernel (lbm_pair.cuh)
+  bool pair = false;
+  int pair_grid = 0;
+  PairParams pq{};
+  void *pair_region = nullptr;
 };
 
 namespace {
@@ -53,6 +59,7 @@ lbm_opts case_opts(const lbm_opts &common, const lbm_case &cs) {
   o.D_ref = cs.D_ref;
   o.rho_in = cs.rho_in;
   o.graph_steps = -1;  // the batch captures its own graphs
+  if (o.kernel == LBM_KERNEL_AUTO) o.kernel = default_kernel(o.storage);
   o.workspace = nullptr;
   o.workspace_bytes = 0;
   return o;
@@ -72,7 +79,7 @@ int batch_sizes(int n, const lbm_case *cases, const lbm_opts *common, std::vecto
     (*sizes)[c] = align_up(b, kAlign);
     sum += (*sizes)[c];
   }
-  *total = sum + desc_bytes(n);
+  *total = sum + desc_bytes(n) + (common->storage == LBM_F32 ? pair_region_bytes(kPairCellsBatch, kPairSlotsBatch, n) : 0);
   return LBM_OK;
 }
 
@@ -111,6 +118,39 @@ int configure_batch(lbm_batch *b, int kernel, int shape, int ctas) {
   return LBM_OK;
 }
 
+// The two-step kernel, for batches that leave the kernel to the library.
+int configure_batch_pair(lbm_batch *b, bool automatic) {
+  b->pair = false;
+  if (!automatic || b->common.storage != LBM_F32 || b->kernel != LBM_KERNEL_TMA) return LBM_OK;
+  const int mrt = b->common.collision == LBM_COLLIDE_MRT ? 1 : 0, n = (int)b->cases.size();
+  CK(pair_batch_f32(0, b->desc, n, mrt, b->pq, b->stream, 1, nullptr));
+  int occ = 0;
+  CK(pair_batch_f32(0, b->desc, n, mrt, b->pq, b->stream, 2, &occ));
+  if (occ < 1) return LBM_OK;
+  std::vector<PairLattice> lattices;
+  for (lbm_ctx *c : b->cases) lattices.push_back({c->nx, c->ny, c->p.bc, &c->geo});
+  const int rc = pair_plan(lattices, b->sms, b->pair_region, kPairCellsBatch, kPairSlotsBatch, b->stream, &b->pq,
+                           &b->pair_grid);
+  if (rc) return rc;
+  b->pair = b->pair_grid > 0;
+  return LBM_OK;
+}
+
+// n steps (even), in passes of two.
+int batch_pair_steps(lbm_batch *b, int64_t n) {
+  const int mrt = b->common.collision == LBM_COLLIDE_MRT ? 1 : 0;
+  while (n > 0) {
+    PairParams q = b->pq;
+    q.pairs = (int)std::min<int64_t>(n / 2, b->pq.pairs);
+    q.parity = b->cur;
+    CK(pair_batch_f32(b->pair_grid, b->desc, (int)b->cases.size(), mrt, q, b->stream, 0, nullptr));
+    b->cur ^= q.pairs & 1;
+    b->launches += 2;
+    n -= 2 * q.pairs;
+  }
+  return LBM_OK;
+}
+
 cudaError_t launch_batch(lbm_batch *b, int parity) {
   const KernelOps *ops = b->cases[0]->ops;
   const int n = (int)b->cases.size();
@@ -125,7 +165,7 @@ int capture_batch_graph(lbm_batch *b) {
     b->graph = nullptr;
   }
   int gs = b->common.graph_steps;
-  if (gs < 0) {
+  if (gs < 0 || b->pair) {
     b->graph_steps = 0;
     return LBM_OK;
   }
@@ -209,6 +249,7 @@ int lbm_batch_create(int ncases, const lbm_case *cases, const lbm_opts *common, 
     b->cases.push_back(ctx);
   }
   b->desc = (CaseDesc *)(base + off);
+  b->pair_region = base + off + desc_bytes(ncases);
   int kernel = common->kernel, shape = default_batch_shape(common->storage);
   int ctas = common->ctas_per_sm > 0 ? common->ctas_per_sm : default_batch_ctas(common->storage);
   if (common->consumer_warps || common->cells_per_thread || common->stages) {
@@ -221,6 +262,9 @@ int lbm_batch_create(int ncases, const lbm_case *cases, const lbm_opts *common, 
   }
   if (kernel == LBM_KERNEL_AUTO) kernel = default_kernel(common->storage);
   rc = configure_batch(b, kernel, shape, ctas);
+  if (rc) return fail(rc);
+  rc = configure_batch_pair(b, common->kernel == LBM_KERNEL_AUTO && !common->consumer_warps && !common->cells_per_thread &&
+                                   !common->stages && common->ctas_per_sm <= 0);
   if (rc) return fail(rc);
   rc = capture_batch_graph(b);
   if (rc) return fail(rc);
@@ -250,6 +294,7 @@ int lbm_batch_init_fields(lbm_batch *b, int c, const double *rho, const double *
   // the batch steps all cases with one parity: bring this case's f*(0) to it
   int rc = lbm_init_fields(ctx, rho, u, v);
   if (rc) return rc;
+  if (b->pair) CK(pair_reset(b->pq, b->stream));
   if (b->cur != 0) {
     CK(cudaMemcpyAsync(ctx->buf[1], ctx->buf[0], (size_t)9 * ctx->plane * ctx->elem, cudaMemcpyDeviceToDevice,
                        b->stream));
@@ -264,6 +309,11 @@ int lbm_batch_step(lbm_batch *b, int64_t n) {
   for (lbm_ctx *c : b->cases)
     if (!c->inited) return LBM_ERR_STATE;
   CK(cudaSetDevice(b->dev));
+  if (b->pair) {
+    const int rc = batch_pair_steps(b, n & ~(int64_t)1);
+    if (rc) return rc;
+    n &= 1;
+  }
   while (n > 0) {
     if (b->graph && b->cur == 0 && n >= b->graph_steps) {
       CK(cudaGraphLaunch(b->graph, b->stream));
@@ -295,6 +345,7 @@ int lbm_batch_set_kernel(lbm_batch *b, int kernel, int ncw, int cpt, int stages,
   CK(cudaSetDevice(b->dev));
   CK(cudaStreamSynchronize(b->stream));
   const int storage = b->common.storage;
+  const bool automatic = kernel == LBM_KERNEL_AUTO && !ncw && !cpt && !stages && ctas_per_sm <= 0;
   int shape = default_batch_shape(storage);
   int ctas = ctas_per_sm > 0 ? ctas_per_sm : default_batch_ctas(storage);
   if (kernel != LBM_KERNEL_DIRECT && (ncw || cpt || stages)) {
@@ -305,7 +356,9 @@ int lbm_batch_set_kernel(lbm_batch *b, int kernel, int ncw, int cpt, int stages,
   } else if (kernel == LBM_KERNEL_AUTO) {
     kernel = default_kernel(storage);
   }
-  const int rc = configure_batch(b, kernel, shape, ctas);
+  int rc = configure_batch(b, kernel, shape, ctas);
+  if (rc) return rc;
+  rc = configure_batch_pair(b, automatic);
   if (rc) return rc;
   return capture_batch_graph(b);
 }

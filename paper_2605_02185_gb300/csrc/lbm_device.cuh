@@ -336,16 +336,16 @@ __device__ __forceinline__ bool plain_span(const StepParams &p, int xa, int xb, 
 //   q >= 1/2:  f*_opp(k)(x) / (2q) + (1 - 1/(2q)) f*_k(x),
 // and, when fxy is given, adds the link's momentum exchange (the population
 // that left along c_opp(k) plus the one that returns) to fxy.
-template <class S, class Fetch, bool INTERP = false, bool COH = false>
-__device__ __forceinline__ void pull(const S *__restrict__ A, const StepParams &p, int xe, int y, uint32_t lm,
-                                     Fetch fetch, typename Store<S>::C h[9], double *fxy = nullptr) {
+// The node's own values come from own(k) -- global memory or a staged copy.
+template <class S, class Fetch, class Own, bool INTERP = false>
+__device__ __forceinline__ void pull_from(const StepParams &p, int xe, int y, uint32_t lm, Fetch fetch, Own own,
+                                          typename Store<S>::C h[9], double *fxy = nullptr) {
   using C = typename Store<S>::C;
-  const size_t own = (size_t)y * p.pitch + xe;
   const C U = (C)p.U;
   C drho_own = (C)0;
   if (p.bc == BC_MOVINGWALL && (y == 0 || y == p.ny - 1)) {
 #pragma unroll
-    for (int k = 0; k < 9; ++k) drho_own += Store<S>::ld(own_ld<COH>(A + (size_t)k * p.plane + own));
+    for (int k = 0; k < 9; ++k) drho_own += own(k);
   }
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
@@ -359,11 +359,11 @@ __device__ __forceinline__ void pull(const S *__restrict__ A, const StepParams &
     }
     if (!inside) {
       if (CY(k) != 0 && p.bc == BC_MOVINGWALL && (unsigned)sy >= (unsigned)p.ny)
-        h[k] = Store<S>::ld(own_ld<COH>(A + (size_t)OPP(k) * p.plane + own)) + (C)(6.0 * WD(k) * CX(k)) * U * drho_own;
+        h[k] = own(OPP(k)) + (C)(6.0 * WD(k) * CX(k)) * U * drho_own;
       else
-        h[k] = Store<S>::ld(own_ld<COH>(A + (size_t)k * p.plane + own));
+        h[k] = own(k);
     } else if (lm & (1u << k)) {
-      const C hi = Store<S>::ld(own_ld<COH>(A + (size_t)OPP(k) * p.plane + own));
+      const C hi = own(OPP(k));
       if constexpr (!INTERP) {
         h[k] = hi;
         if (CX(k) != 0) h[k] += (C)(-6.0 * WD(k) * CX(k)) * U;
@@ -378,7 +378,7 @@ __device__ __forceinline__ void pull(const S *__restrict__ A, const StepParams &
           wref = (C)1;
         } else {
           const C a = (C)(0.5f / q);
-          v = a * hi + ((C)1 - a) * Store<S>::ld(own_ld<COH>(A + (size_t)k * p.plane + own));
+          v = a * hi + ((C)1 - a) * own(k);
           wref = a;
         }
         if (CX(k) != 0) v += (C)(-6.0 * WD(k) * CX(k)) * U * wref;
@@ -393,6 +393,25 @@ __device__ __forceinline__ void pull(const S *__restrict__ A, const StepParams &
       h[k] = fetch(k, sx, sy);
     }
   }
+}
+
+template <class S, class Fetch, bool INTERP = false, bool COH = false>
+__device__ __forceinline__ void pull(const S *__restrict__ A, const StepParams &p, int xe, int y, uint32_t lm,
+                                     Fetch fetch, typename Store<S>::C h[9], double *fxy = nullptr) {
+  const size_t at = (size_t)y * p.pitch + xe;
+  auto own = [&](int k) -> typename Store<S>::C { return Store<S>::ld(own_ld<COH>(A + (size_t)k * p.plane + at)); };
+  pull_from<S, Fetch, decltype(own), INTERP>(p, xe, y, lm, fetch, own, h, fxy);
+}
+
+// Zou-He velocity inlet (U, 0): unknowns f2, f6, f9 from the six others.
+template <class C>
+__device__ __forceinline__ void inlet(C h[9], C U) {
+  const C drho = (h[0] + h[2] + h[4] + (C)2 * (h[3] + h[6] + h[7])) / ((C)1 - U);
+  const C ru = drho * U;
+  const C hh = (C)0.5 * (h[2] - h[4]);
+  h[1] = h[3] + ((C)2 / (C)3) * ru;
+  h[5] = h[7] - hh + ru / (C)6;
+  h[8] = h[6] + hh + ru / (C)6;
 }
 
 // Boundary corrections after streaming (Section 2.3), in the order top row,
@@ -432,14 +451,7 @@ __device__ __forceinline__ void boundaries(C h[9], int xe, int y, const StepPara
       }
     }
   }
-  if (xe == 0) {  // Zou-He velocity inlet (U, 0): unknowns f2, f6, f9
-    const C drho = (h[0] + h[2] + h[4] + (C)2 * (h[3] + h[6] + h[7])) / ((C)1 - U);
-    const C ru = drho * U;
-    const C hh = (C)0.5 * (h[2] - h[4]);
-    h[1] = h[3] + ((C)2 / (C)3) * ru;
-    h[5] = h[7] - hh + ru / (C)6;
-    h[8] = h[6] + hh + ru / (C)6;
-  }
+  if (xe == 0) inlet<C>(h, U);
 }
 
 // ---- lane arithmetic -------------------------------------------------------
@@ -780,6 +792,17 @@ __device__ __forceinline__ void named_bar(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
+// ---- two-step kernel: the split of the lattices over its warps ---------------
+struct PairParams {
+  const int4 *cells;        // (case << 16 | window, first row, past the last row, force slot or -1)
+  const int *deps;          // [ncells][32] the cells a cell exchanges nodes with, then -1
+  unsigned *flags;          // [ncells] passes done since the flags were last cleared
+  double2 *slots;           // [2 pairs][nslots] force partials of the cells that own links
+  const int2 *case_slots;   // batch: slots [x, y) of each case
+  int ncells, nslots;
+  int pairs, parity;        // passes of this launch (on the host: at most); batch: the buffer it starts from
+};
+
 // ---- multi-step kernel: per-row completion counters ------------------------
 // rows_done[y] counts the row tiles of row y that finished a step, over the
 // launches since the counters were last cleared: when a launch starts, every
@@ -796,6 +819,9 @@ __device__ __forceinline__ unsigned ld_relaxed_gpu(const unsigned *p) {
   unsigned v;
   asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
+}
+__device__ __forceinline__ void st_relaxed_gpu(unsigned *p, unsigned v) {
+  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 __device__ __forceinline__ void red_relaxed_gpu_add(unsigned *p, unsigned v) {
   asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");

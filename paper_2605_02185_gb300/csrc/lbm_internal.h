@@ -10,6 +10,7 @@ namespace gblbm {
 struct StepParams;
 struct CaseDesc;
 struct WaveParams;
+struct PairParams;
 
 // Launchers of one storage type.  All launches are asynchronous on `st`.
 struct KernelOps {
@@ -127,6 +128,21 @@ struct WaveShape {
 constexpr WaveShape kWaveShapes[] = {GBLBM_WAVE_SHAPES(GBLBM_SHAPE_ENTRY)};
 #undef GBLBM_SHAPE_ENTRY
 constexpr int kNumWaveShapes = (int)(sizeof(kWaveShapes) / sizeof(kWaveShapes[0]));
+// ---- the two-step kernel (lbm_pair.cuh, lbm_pair.cu), float storage ----------
+constexpr int kPairCols = 64;            // columns a warp stages
+constexpr int kPairOut = kPairCols - 4;  // columns it yields, from the third on
+constexpr int kPairMargin = 4;           // window w starts at column 60 w - 4
+constexpr int kPairWarps = 16;           // warps per CTA, one CTA per SM
+constexpr int kPairStages = 5;           // staged rows per warp
+constexpr int kPairMax = 32;             // passes (of two steps) per launch
+// mode 0: launch q.pairs passes from buf0 (on even passes) into buf1, and the
+// sums of their forces; 1: set the shared-memory limit; 2: resident CTAs per SM
+// into *occ.
+cudaError_t pair_f32(int grid, void *buf0, void *buf1, const StepParams &p, const PairParams &q, cudaStream_t st,
+                     int mode, int *occ);
+cudaError_t pair_batch_f32(int grid, const CaseDesc *cases, int ncases, int mrt, const PairParams &q, cudaStream_t st,
+                           int mode, int *occ);
+
 // Steps per launch of the multi-step kernel.
 constexpr int kWaveSteps = 64;
 #define GBLBM_SHAPE_ENTRY(id, a, b, c) {a, b, c},

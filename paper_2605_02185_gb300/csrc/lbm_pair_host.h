@@ -1,0 +1,34 @@
+// lbm_pair_host.h -- host side of the two-step kernel: the cells its warps work
+// on, shared by single lattices and batches.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <vector>
+
+#include "lbm_ctx.h"
+#include "lbm_internal.h"
+
+namespace gblbm {
+
+// Capacities of a workspace region for `cases` lattices; a plan that needs more
+// leaves its lattices to the one-step kernels.
+constexpr int kPairCellsSingle = 4096, kPairSlotsSingle = 512;
+constexpr int kPairCellsBatch = 8192, kPairSlotsBatch = 4096;
+size_t pair_region_bytes(int cells, int slots, int cases);
+
+struct PairLattice {
+  int nx, ny, bc;
+  const Geometry *geo;
+};
+
+// Split the lattices over the warps of `sms` SMs, upload the tables into `region`
+// (pair_region_bytes() of it) on `st` and fill q (q->pairs: the most passes of a
+// launch) and *grid.  LBM_OK with *grid = 0
+// where the kernel does not take them.
+int pair_plan(const std::vector<PairLattice> &lattices, int sms, void *region, int cells_cap, int slots_cap,
+              cudaStream_t st, PairParams *q, int *grid);
+// Clear the cells' flags (a new state; a launch that gave up left them uneven).
+cudaError_t pair_reset(const PairParams &q, cudaStream_t st);
+
+}  // namespace gblbm
