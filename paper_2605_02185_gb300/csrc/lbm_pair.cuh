@@ -88,19 +88,6 @@ __device__ __forceinline__ void set_elem(float2 &v, int j, float s) {
   else v.x = s;
 }
 
-// A sum of floats kept to twice their precision (two-sum, Knuth): this chip does
-// few double operations, so a row's link populations are added here and the row's
-// sum goes to the double total.  (Both are exact for populations within a factor
-// 2^24 of each other, so the order of the sum does not show.)
-struct Sum2 {
-  float hi = 0.f, lo = 0.f;
-  __device__ __forceinline__ void add(float v) {
-    const float t = hi + v, z = t - hi;
-    lo += (hi - (t - z)) + (v - z);
-    hi = t;
-  }
-};
-
 // The wall rules of boundaries() for a node of the bottom or top row.
 __device__ __forceinline__ void pair_wall(int bc, bool bottom, float U, float (&v)[9]) {
   if (bc == BC_FREESLIP) {
@@ -255,7 +242,9 @@ __global__ void __launch_bounds__(NW * 32, 1)
     const Coef<LP2> cf = make_coef<LP2>(p);
     const float U = (float)p.U;
     uint32_t worst = 0;                             // largest |u|^2 seen, as bits
-    double fx[2] = {0.0, 0.0}, fy[2] = {0.0, 0.0};  // this lane's links, per stage
+    // this lane's links, per stage: a row's links are added in float pairs, the
+    // row's sum goes to the double total
+    double fx[2] = {0.0, 0.0}, fy[2] = {0.0, 0.0};
     int st = 0;                                     // stage of the current row's tile
     const bool map_cols = p.lx0 < base + kPairCols && p.lx0 + p.lw > base;  // the window meets the link map
     const bool has_inlet = base <= 0, has_outlet = base + kPairCols >= nx;
