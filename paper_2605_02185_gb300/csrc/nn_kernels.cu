@@ -422,6 +422,111 @@ __global__ void upsample2_bwd_kernel(const bf16 *__restrict__ gy, int gs, bf16 *
   }
 }
 
+// ---- the same, eight channels (16 bytes) per access --------------------------
+// The kernels above move two bytes per thread and access behind three 64-bit
+// divisions and ran at 2-10 % of the memory bandwidth.  Here a block covers 256
+// vectors of one row of the small image (blockIdx.x: the row, over all samples),
+// a thread takes one of its vectors and the 2 x 2 vectors of the large image
+// around it; the large image's row is 2 r because its height is twice the small
+// one's.  Taken when channels, strides and pointers are multiples of 16 bytes.
+// Training shape (4 x 800 x 1600, all levels), before and now: upsample 3.97 ->
+// 0.22 ms, its gradient and pooling 1.79 -> 0.41, pooling's gradient 2.37 -> 0.42.
+struct Vec8 {
+  __nv_bfloat162 v[4];
+};
+__device__ __forceinline__ Vec8 ldv(const bf16 *p) {
+  const uint4 t = *reinterpret_cast<const uint4 *>(p);
+  Vec8 r;
+  r.v[0] = *reinterpret_cast<const __nv_bfloat162 *>(&t.x);
+  r.v[1] = *reinterpret_cast<const __nv_bfloat162 *>(&t.y);
+  r.v[2] = *reinterpret_cast<const __nv_bfloat162 *>(&t.z);
+  r.v[3] = *reinterpret_cast<const __nv_bfloat162 *>(&t.w);
+  return r;
+}
+__device__ __forceinline__ void stv(bf16 *p, const Vec8 &a) {
+  uint4 t;
+  t.x = *reinterpret_cast<const uint32_t *>(&a.v[0]);
+  t.y = *reinterpret_cast<const uint32_t *>(&a.v[1]);
+  t.z = *reinterpret_cast<const uint32_t *>(&a.v[2]);
+  t.w = *reinterpret_cast<const uint32_t *>(&a.v[3]);
+  *reinterpret_cast<uint4 *>(p) = t;
+}
+// scale * (((a + b) + c) + d), in float as the kernels above
+__device__ __forceinline__ Vec8 sum4(const Vec8 &a, const Vec8 &b, const Vec8 &c, const Vec8 &d, float scale) {
+  Vec8 r;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const float2 x = __bfloat1622float2(a.v[e]), y = __bfloat1622float2(b.v[e]), z = __bfloat1622float2(c.v[e]),
+                 w = __bfloat1622float2(d.v[e]);
+    r.v[e] = __floats2bfloat162_rn(scale * (x.x + y.x + z.x + w.x), scale * (x.y + y.y + z.y + w.y));
+  }
+  return r;
+}
+
+// W: width of the small image; c8: vectors per pixel
+__global__ void __launch_bounds__(256) upsample2_vec_kernel(const bf16 *__restrict__ x, int xs, bf16 *__restrict__ y, int ys,
+                                                           int W, int c8) {
+  const int i = blockIdx.y * 256 + threadIdx.x;
+  if (i >= W * c8) return;
+  const int w = i / c8, c = 8 * (i - w * c8);
+  const size_t r = blockIdx.x;
+  const Vec8 v = ldv(x + (r * W + w) * xs + c);
+  bf16 *o = y + (4 * r * W + 2 * w) * ys + c;
+  stv(o, v);
+  stv(o + ys, v);
+  o += (size_t)2 * W * ys;
+  stv(o, v);
+  stv(o + ys, v);
+}
+
+// y = scale * the sum over the 2 x 2 parents' children (pooling: 1/4; the
+// gradient of upsampling: 1)
+__global__ void __launch_bounds__(256) sum2x2_vec_kernel(const bf16 *__restrict__ x, int xs, bf16 *__restrict__ y, int ys,
+                                                        int W, int c8, float scale) {
+  const int i = blockIdx.y * 256 + threadIdx.x;
+  if (i >= W * c8) return;
+  const int w = i / c8, c = 8 * (i - w * c8);
+  const size_t r = blockIdx.x;
+  const bf16 *a = x + (4 * r * W + 2 * w) * xs + c, *b = a + (size_t)2 * W * xs;
+  stv(y + (r * W + w) * ys + c, sum4(ldv(a), ldv(a + xs), ldv(b), ldv(b + xs), scale));
+}
+
+__global__ void __launch_bounds__(256) avgpool2_bwd_vec_kernel(const bf16 *__restrict__ gy, int gs, bf16 *__restrict__ gx,
+                                                              int gxs, const bf16 *__restrict__ mask, int ms, int W, int c8,
+                                                              int accumulate) {
+  const int i = blockIdx.y * 256 + threadIdx.x;
+  if (i >= W * c8) return;
+  const int w = i / c8, c = 8 * (i - w * c8);
+  const size_t r = blockIdx.x;
+  const Vec8 g = ldv(gy + (r * W + w) * gs + c);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const size_t pix = 4 * r * W + 2 * w + (q & 1) + (size_t)(q >> 1) * 2 * W;
+    bf16 *o = gx + pix * gxs + c;
+    Vec8 m, old, out;
+    if (mask) m = ldv(mask + pix * ms + c);
+    if (accumulate) old = ldv(o);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      float2 v = __bfloat1622float2(g.v[e]);
+      v.x *= 0.25f;
+      v.y *= 0.25f;
+      if (mask) {
+        const float2 k = __bfloat1622float2(m.v[e]);
+        if (!(k.x > 0.f)) v.x = 0.f;
+        if (!(k.y > 0.f)) v.y = 0.f;
+      }
+      if (accumulate) {
+        const float2 k = __bfloat1622float2(old.v[e]);
+        v.x += k.x;
+        v.y += k.y;
+      }
+      out.v[e] = __floats2bfloat162_rn(v.x, v.y);
+    }
+    stv(o, out);
+  }
+}
+
 // loss partials: sum over elements of wgt * (pred - target)^2; grad = 2 wgt (pred - target) * scale
 __global__ void mse_kernel(const bf16 *__restrict__ pred, int ps, const float *__restrict__ target,
                            const float *__restrict__ weight, bf16 *__restrict__ grad, int gs, long long P, int C,
@@ -515,6 +620,17 @@ int g_conv_impl = GBNN_IMPL_AUTO;
 int grid_for(long long n) {
   long long b = (n + 255) / 256;
   return (int)(b < 1 ? 1 : (b > 65535 * 16 ? 65535 * 16 : b));
+}
+
+// The vector kernels take 16-byte channels, strides and pointers; W is the small
+// image's width, rows = N * its height.
+bool vec_ok(int C, int s0, int s1, int s2, const void *p0, const void *p1, const void *p2, long long rows, int W) {
+  return C > 0 && C % 8 == 0 && s0 % 8 == 0 && s1 % 8 == 0 && s2 % 8 == 0 &&
+         (((uintptr_t)p0 | (uintptr_t)p1 | (uintptr_t)p2) & 15) == 0 && rows > 0 && rows <= 0x7fffffff && W > 0 &&
+         (long long)W * (C / 8) <= 65535ll * 256;
+}
+dim3 vec_grid(long long rows, int W, int C) {
+  return dim3((unsigned)rows, (unsigned)(((long long)W * (C / 8) + 255) / 256));
 }
 
 int err(cudaError_t e) { return e == cudaSuccess ? 0 : -2; }
@@ -615,6 +731,11 @@ int gbnn_conv3x3_wgrad(const void *x, int x_cstride, const void *gy, int gy_cstr
 
 int gbnn_avgpool2(const void *x, int x_cstride, void *y, int y_cstride, int N, int H, int W, int C, void *stream) {
   if (H % 2 || W % 2) return -1;
+  if (vec_ok(C, x_cstride, y_cstride, 0, x, y, nullptr, (long long)N * (H / 2), W / 2)) {
+    sum2x2_vec_kernel<<<vec_grid((long long)N * (H / 2), W / 2, C), 256, 0, (cudaStream_t)stream>>>(
+        (const bf16 *)x, x_cstride, (bf16 *)y, y_cstride, W / 2, C / 8, 0.25f);
+    return err(cudaGetLastError());
+  }
   const long long n = (long long)N * (H / 2) * (W / 2) * C;
   avgpool2_kernel<<<grid_for(n), 256, 0, (cudaStream_t)stream>>>((const bf16 *)x, x_cstride, (bf16 *)y, y_cstride, N, H,
                                                                   W, C);
@@ -624,6 +745,11 @@ int gbnn_avgpool2(const void *x, int x_cstride, void *y, int y_cstride, int N, i
 int gbnn_avgpool2_bwd(const void *gy, int gy_cstride, void *gx, int gx_cstride, const void *mask, int mask_cstride,
                       int N, int H, int W, int C, int accumulate, void *stream) {
   if (H % 2 || W % 2) return -1;
+  if (vec_ok(C, gy_cstride, gx_cstride, mask ? mask_cstride : 0, gy, gx, mask, (long long)N * (H / 2), W / 2)) {
+    avgpool2_bwd_vec_kernel<<<vec_grid((long long)N * (H / 2), W / 2, C), 256, 0, (cudaStream_t)stream>>>(
+        (const bf16 *)gy, gy_cstride, (bf16 *)gx, gx_cstride, (const bf16 *)mask, mask_cstride, W / 2, C / 8, accumulate);
+    return err(cudaGetLastError());
+  }
   const long long n = (long long)N * H * W * C;
   avgpool2_bwd_kernel<<<grid_for(n), 256, 0, (cudaStream_t)stream>>>((const bf16 *)gy, gy_cstride, (bf16 *)gx,
                                                                       gx_cstride, (const bf16 *)mask, mask_cstride, N,
@@ -632,6 +758,11 @@ int gbnn_avgpool2_bwd(const void *gy, int gy_cstride, void *gx, int gx_cstride, 
 }
 
 int gbnn_upsample2(const void *x, int x_cstride, void *y, int y_cstride, int N, int H, int W, int C, void *stream) {
+  if (vec_ok(C, x_cstride, y_cstride, 0, x, y, nullptr, (long long)N * H, W)) {
+    upsample2_vec_kernel<<<vec_grid((long long)N * H, W, C), 256, 0, (cudaStream_t)stream>>>(
+        (const bf16 *)x, x_cstride, (bf16 *)y, y_cstride, W, C / 8);
+    return err(cudaGetLastError());
+  }
   const long long n = (long long)N * 4 * H * W * C;
   upsample2_kernel<<<grid_for(n), 256, 0, (cudaStream_t)stream>>>((const bf16 *)x, x_cstride, (bf16 *)y, y_cstride, N,
                                                                    H, W, C);
@@ -640,6 +771,11 @@ int gbnn_upsample2(const void *x, int x_cstride, void *y, int y_cstride, int N, 
 
 int gbnn_upsample2_bwd(const void *gy, int gy_cstride, void *gx, int gx_cstride, int N, int H, int W, int C,
                        void *stream) {
+  if (vec_ok(C, gy_cstride, gx_cstride, 0, gy, gx, nullptr, (long long)N * H, W)) {
+    sum2x2_vec_kernel<<<vec_grid((long long)N * H, W, C), 256, 0, (cudaStream_t)stream>>>(
+        (const bf16 *)gy, gy_cstride, (bf16 *)gx, gx_cstride, W, C / 8, 1.f);
+    return err(cudaGetLastError());
+  }
   const long long n = (long long)N * H * W * C;
   upsample2_bwd_kernel<<<grid_for(n), 256, 0, (cudaStream_t)stream>>>((const bf16 *)gy, gy_cstride, (bf16 *)gx,
                                                                        gx_cstride, N, H, W, C);

