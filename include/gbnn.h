@@ -35,7 +35,8 @@ extern "C" {
  *   multiples of 32, cout <= 256, strides multiples of 8, x and gy 16-byte
  *   aligned.
  * GBNN_IMPL_MMA_SYNC: the warp-level m16n8k16 kernels (every shape).
- * GBNN_IMPL_AUTO (default): tcgen05 where the shape is taken, else mma.sync.
+ * GBNN_IMPL_AUTO (default): tcgen05 where the shape is taken (here also 8 -> 32
+ *   and 32 -> 8 channels, forward and input gradient), else mma.sync.
  * gbnn_set_conv_impl applies to every later convolution call of the process
  * (not thread-safe); with GBNN_IMPL_TCGEN05 a shape it does not take returns
  * -1.  gbnn_status reads (and with reset != 0 clears) the device status word

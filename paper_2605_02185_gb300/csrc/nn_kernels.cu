@@ -658,7 +658,7 @@ int gbnn_conv3x3_fwd(const void *x, int x_cstride, const void *w, const float *b
   const cudaStream_t st = (cudaStream_t)stream;
   if (g_conv_impl != GBNN_IMPL_MMA_SYNC) {
     const int rc = gbnn_tc::conv_fwd(x, x_cstride, w, bias, y, y_cstride, mask, mask_cstride, N, H, W, cin, cout, relu,
-                                     st);
+                                     g_conv_impl == GBNN_IMPL_AUTO, st);
     if (rc != gbnn_tc::kNotEligible) return rc;
     if (g_conv_impl == GBNN_IMPL_TCGEN05) return -1;  // required, but this shape is not taken
   }

@@ -705,6 +705,8 @@ cudaError_t launch(const CUtensorMap &tx, const CUtensorMap &tw, const float *bi
   return cudaGetLastError();
 }
 
+#include "nn_rows.cuh"
+
 bool eligible(int cin, int cout, int xs, int ys, const void *x, const void *w, const void *y, const void *mask,
               int ms) {
   if (cin % 32 || cout % 32 || cout > 512 || xs % 8 || ys % 8) return false;
@@ -715,7 +717,9 @@ bool eligible(int cin, int cout, int xs, int ys, const void *x, const void *w, c
 }
 
 int conv_fwd(const void *x, int xs, const void *w, const float *bias, void *y, int ys, const void *mask, int ms, int N,
-             int H, int W, int cin, int cout, int relu, cudaStream_t st) {
+             int H, int W, int cin, int cout, int relu, bool eight, cudaStream_t st) {
+  const int rc = conv_rows(x, xs, w, bias, y, ys, mask, ms, N, H, W, cin, cout, relu, eight, st);
+  if (rc != kNotEligible) return rc;
   if (!eligible(cin, cout, xs, ys, x, w, y, mask, ms)) return kNotEligible;
   PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
   if (!enc) return -2;

@@ -9,10 +9,10 @@ namespace gbnn_tc {
 constexpr int kNotEligible = 1;  // shape or alignment the tensor-core kernels do not take
 
 // y = act(conv3x3(x, w) + bias) on the tensor cores (arguments as
-// gbnn_conv3x3_fwd).  0 on success, kNotEligible (nothing launched), or -2
+// gbnn_conv3x3_fwd; eight: also layers of 8 input or output channels).  0 on success, kNotEligible (nothing launched), or -2
 // for a CUDA error.
 int conv_fwd(const void *x, int xs, const void *w, const float *bias, void *y, int ys, const void *mask, int ms, int N,
-             int H, int W, int cin, int cout, int relu, cudaStream_t st);
+             int H, int W, int cin, int cout, int relu, bool eight, cudaStream_t st);
 
 // gw += dL/dw (and gb += dL/db if gb) on the tensor cores (arguments as
 // gbnn_conv3x3_wgrad).  0, kNotEligible (nothing launched) or -2.
