@@ -263,6 +263,7 @@ __global__ void __launch_bounds__(WG_THREADS) conv_wgrad_kernel(const bf16 *__re
 constexpr int W9_PX = 64;
 constexpr int W9_CP = 40;  // padded channel stride (conflict-free ldmatrix rows)
 constexpr int W9_THREADS = 288;
+constexpr int W9_XV = (3 * (W9_PX + 2) * 4 + W9_THREADS - 1) / W9_THREADS;  // x vectors per thread and segment
 
 struct W9Smem {
   bf16 g[W9_PX][W9_CP];              // [pixel][o]
@@ -293,28 +294,42 @@ __global__ void __launch_bounds__(W9_THREADS) conv_wgrad9_kernel(const bf16 *__r
 #pragma unroll
       for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.f;
 
-  for (long long sg = s_begin; sg < s_end; ++sg) {
+  // The next segment's vectors travel to registers while the tensor cores work
+  // on this one: without that the block waited for memory at every segment
+  // (4 x 800 x 1600: 867 and 754 us for 8 output and 8 input channels, 425 now).
+  uint4 gv, xv[W9_XV];
+  auto fetch = [&](long long sg) {
     const int w0 = (int)(sg % spr) * W9_PX;
     const long long r = sg / spr;
     const int h = (int)(r % H), n = (int)(r / H);
-    for (int i = tid; i < W9_PX * 4; i += W9_THREADS) {  // gy: 64 pixels x 32 channels
-      const int v = i & 3, px = i >> 2;
-      uint4 val = make_uint4(0, 0, 0, 0);
+    gv = make_uint4(0, 0, 0, 0);
+    if (tid < W9_PX * 4) {  // gy: 64 pixels x 32 channels
+      const int v = tid & 3, px = tid >> 2;
       if (w0 + px < W && o0 + v * 8 < cout)
-        val = *reinterpret_cast<const uint4 *>(gy + (((size_t)n * H + h) * W + w0 + px) * gs + o0 + v * 8);
-      *reinterpret_cast<uint4 *>(&sm.g[px][v * 8]) = val;
+        gv = *reinterpret_cast<const uint4 *>(gy + (((size_t)n * H + h) * W + w0 + px) * gs + o0 + v * 8);
     }
-    for (int i = tid; i < 3 * (W9_PX + 2) * 4; i += W9_THREADS) {  // x: 3 rows x 66 pixels x 32 channels
+#pragma unroll
+    for (int e = 0; e < W9_XV; ++e) {  // x: 3 rows x 66 pixels x 32 channels
+      const int i = tid + e * W9_THREADS;
       const int v = i & 3, px = (i >> 2) % (W9_PX + 2), rr = (i >> 2) / (W9_PX + 2);
       const int hh = h + rr - 1, ww = w0 + px - 1;
-      uint4 val = make_uint4(0, 0, 0, 0);
-      if (hh >= 0 && hh < H && ww >= 0 && ww < W && c0 + v * 8 < cin)
-        val = *reinterpret_cast<const uint4 *>(x + (((size_t)n * H + hh) * W + ww) * xs + c0 + v * 8);
-      *reinterpret_cast<uint4 *>(&sm.xs[rr][px][v * 8]) = val;
+      xv[e] = make_uint4(0, 0, 0, 0);
+      if (rr < 3 && hh >= 0 && hh < H && ww >= 0 && ww < W && c0 + v * 8 < cin)
+        xv[e] = *reinterpret_cast<const uint4 *>(x + (((size_t)n * H + hh) * W + ww) * xs + c0 + v * 8);
+    }
+  };
+  if (s_begin < s_end) fetch(s_begin);
+  for (long long sg = s_begin; sg < s_end; ++sg) {
+    if (tid < W9_PX * 4) *reinterpret_cast<uint4 *>(&sm.g[tid >> 2][(tid & 3) * 8]) = gv;
+#pragma unroll
+    for (int e = 0; e < W9_XV; ++e) {
+      const int i = tid + e * W9_THREADS, px = (i >> 2) % (W9_PX + 2), rr = (i >> 2) / (W9_PX + 2);
+      if (rr < 3) *reinterpret_cast<uint4 *>(&sm.xs[rr][px][(i & 3) * 8]) = xv[e];
     }
     __syncthreads();
-    if (do_bias && tid < 32)
-      for (int px = 0; px < W9_PX; ++px) bsum += __bfloat162float(sm.g[px][tid]);
+    if (sg + 1 < s_end) fetch(sg + 1);
+    if (do_bias)  // lane: channel; the warps share the pixels
+      for (int px = warp; px < W9_PX; px += 9) bsum += __bfloat162float(sm.g[px][lane]);
 #pragma unroll
     for (int kk = 0; kk < W9_PX; kk += 16) {
       const int q = lane >> 3, rw = lane & 7;
@@ -352,7 +367,7 @@ __global__ void __launch_bounds__(W9_THREADS) conv_wgrad9_kernel(const bf16 *__r
         atomicAdd(dst + 1, acc[mt][nt][2 * hf + 1]);
       }
     }
-  if (do_bias && tid < 32 && o0 + tid < cout) atomicAdd(gb + o0 + tid, bsum);
+  if (do_bias && o0 + lane < cout) atomicAdd(gb + o0 + lane, bsum);
 }
 
 // wf[c, dy, dx, o] = w[o, 2-dy, 2-dx, c]
