@@ -1158,107 +1158,6 @@ __global__ void init_device_kernel(S *__restrict__ A, StepParams p, const float 
   }
 }
 
-// The same for float, half and bfloat16 storage in float pairs (about 46 bits):
-// the double form's ~225 double operations a node bound it (1600 x 800: 443 us).
-// h_k / w_k = rho dP_k + drho P_k(U, 0) - n_k, with dP_k = P_k(u, v) - P_k(U, 0) =
-// 3 s + 9/2 s t - 3/2 q formed from small quantities (s = c.(du, v), t =
-// c.(u + U, v), q = du (u + U) + v^2), so that no term cancels, and n_k the
-// non-equilibrium part, which like 9/2 s t - 3/2 q is the same for opposite k.
-struct DF {
-  float hi, lo;
-};
-__device__ __forceinline__ DF df_fast(float a, float b) {  // |a| >= |b|
-  const float t = __fadd_rn(a, b);
-  return {t, __fsub_rn(b, __fsub_rn(t, a))};
-}
-__device__ __forceinline__ DF df_sum(float a, float b) {
-  const float t = __fadd_rn(a, b), z = __fsub_rn(t, a);
-  return {t, __fadd_rn(__fsub_rn(a, __fsub_rn(t, z)), __fsub_rn(b, z))};
-}
-__device__ __forceinline__ DF operator+(DF a, DF b) {
-  const DF t = df_sum(a.hi, b.hi);
-  return df_fast(t.hi, __fadd_rn(t.lo, __fadd_rn(a.lo, b.lo)));
-}
-__device__ __forceinline__ DF operator-(DF a) { return {-a.hi, -a.lo}; }
-__device__ __forceinline__ DF operator-(DF a, DF b) { return a + (-b); }
-__device__ __forceinline__ DF operator*(DF a, DF b) {
-  const float p = __fmul_rn(a.hi, b.hi);
-  return df_fast(p, __fadd_rn(__fmaf_rn(a.hi, b.hi, -p), __fmaf_rn(a.hi, b.lo, __fmul_rn(a.lo, b.hi))));
-}
-__device__ __forceinline__ DF operator*(float a, DF b) {
-  const float p = __fmul_rn(a, b.hi);
-  return df_fast(p, __fmaf_rn(a, b.lo, __fmaf_rn(a, b.hi, -p)));
-}
-__host__ __device__ constexpr DF df_of(double v) { return {(float)v, (float)(v - (double)(float)v)}; }
-
-struct InitConsts {
-  DF U, p0[3], n3;  // P_k(U, 0) for c_kx = -1, 0, 1; 3 (tau - 1)
-};
-
-template <class S>
-__global__ void __launch_bounds__(256) init_device_pair_kernel(S *__restrict__ A, const __grid_constant__ StepParams p,
-                                                               const __grid_constant__ InitConsts c,
-                                                               const float *__restrict__ rho, const float *__restrict__ u,
-                                                               const float *__restrict__ v, int with_noneq) {
-  const unsigned i = blockIdx.x * 256u + threadIdx.x;
-  if (i >= (unsigned)p.nx * (unsigned)p.ny) return;
-  const int y = (int)(i / (unsigned)p.nx), x = (int)(i - (unsigned)y * (unsigned)p.nx);
-  S *o = A + (size_t)y * p.pitch + x;
-  if (link_mask(p, x, y) & LM_SOLID) {
-#pragma unroll
-    for (int k = 0; k < 9; ++k) o[(size_t)k * p.plane] = Store<S>::st(0);
-    return;
-  }
-  const float r = rho[i], ux = u[i], uy = v[i];
-  const DF dr = df_sum(r, -1.f), vy = {uy, 0.f};
-  const DF du = df_sum(ux, -c.U.hi) + DF{-c.U.lo, 0.f}, su = df_sum(ux, c.U.hi) + DF{c.U.lo, 0.f};
-  const DF q15 = 1.5f * (du * su + vy * vy);
-  DF gxx = {0.f, 0.f}, gyy = gxx, gxy = gxx;  // du/dx, dv/dy, du/dy + dv/dx, times 3 (tau - 1) rho
-  if (with_noneq) {
-    auto diff = [&](const float *f, int ddx, int ddy) -> DF {  // as diff1
-      const bool lo = fluid_at(p, x - ddx, y - ddy), hi = fluid_at(p, x + ddx, y + ddy);
-      const long long step = (long long)ddy * p.nx + ddx;
-      const float fc = f[i], fl = lo ? f[(long long)i - step] : fc, fh = hi ? f[(long long)i + step] : fc;
-      return (lo && hi ? 0.5f : 1.f) * df_sum(fh, -fl);
-    };
-    const DF n = r * c.n3;
-    gxx = n * diff(u, 1, 0);
-    gyy = n * diff(v, 0, 1);
-    gxy = n * (diff(u, 0, 1) + diff(v, 1, 0));
-  }
-  constexpr DF third = df_of(1.0 / 3.0);
-  const DF trace = third * (gxx + gyy);
-  auto put = [&](int k, DF dp, DF n) {
-    const DF h = df_of(WD(k)) * ((r * dp + dr * c.p0[CX(k) + 1]) - n);
-    o[(size_t)k * p.plane] = Store<S>::st(h.hi);
-  };
-  put(0, -q15, -trace);
-#pragma unroll
-  for (int k = 1; k < 9; ++k) {
-    if (k == 3 || k == 4 || k == 7 || k == 8) continue;  // with their opposites 1, 2, 5, 6
-    DF s, t, n;
-    if (k == 1) {
-      s = du;
-      t = su;
-      n = gxx - trace;
-    } else if (k == 2) {
-      s = t = vy;
-      n = gyy - trace;
-    } else if (k == 5) {
-      s = du + vy;
-      t = su + vy;
-      n = gxx + gyy - trace + gxy;
-    } else {
-      s = vy - du;
-      t = vy - su;
-      n = gxx + gyy - trace - gxy;
-    }
-    const DF even = 4.5f * (s * t) - q15, odd = 3.f * s;
-    put(k, even + odd, n);
-    put(OPP(k), even - odd, n);
-  }
-}
-
 // ---- Eq. 14 force of the stored f*, one CTA, fixed order -----------------
 template <class S>
 __global__ void __launch_bounds__(256) force_kernel(const S *__restrict__ A, StepParams p) {
@@ -1668,14 +1567,6 @@ struct Launch {
   static cudaError_t init_device(void *A, const StepParams &p, const float *r, const float *u, const float *v,
                                  int with_noneq, double tau, cudaStream_t st) {
     const long long n = (long long)p.nx * p.ny;
-    if constexpr (std::is_same<typename Store<S>::C, float>::value) {
-      InitConsts c;
-      c.U = df_of(p.U);
-      for (int cx = -1; cx <= 1; ++cx) c.p0[cx + 1] = df_of(1.0 + 3.0 * cx * p.U + (4.5 * cx * cx - 1.5) * p.U * p.U);
-      c.n3 = df_of(3.0 * (tau - 1.0));
-      init_device_pair_kernel<S><<<(unsigned)((n + 255) / 256), 256, 0, st>>>((S *)A, p, c, r, u, v, with_noneq);
-      return cudaGetLastError();
-    }
     const int blocks = (int)((n + 255) / 256 < 65535 * 8 ? (n + 255) / 256 : 65535 * 8);
     init_device_kernel<S><<<blocks > 0 ? blocks : 1, 256, 0, st>>>((S *)A, p, r, u, v, with_noneq, tau);
     return cudaGetLastError();
