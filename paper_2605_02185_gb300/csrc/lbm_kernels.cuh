@@ -1125,8 +1125,11 @@ __global__ void init_device_kernel(S *__restrict__ A, StepParams p, const float 
                                    const float *__restrict__ u, const float *__restrict__ v, int with_noneq,
                                    double tau) {
   const long long n = (long long)p.nx * p.ny;
+  double rp[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) rp[k] = ref_pop(k, p.U);
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const int x = (int)(i % p.nx), y = (int)(i / p.nx);
+    const int y = (int)(i / p.nx), x = (int)(i - (long long)y * p.nx);
     const uint32_t lm = link_mask(p, x, y);
     const size_t o = (size_t)y * p.pitch + x;
     if (lm & LM_SOLID) {
@@ -1135,7 +1138,7 @@ __global__ void init_device_kernel(S *__restrict__ A, StepParams p, const float 
       continue;
     }
     const double r = rho[i], ux = u[i], uy = v[i];
-    const double uu = ux * ux + uy * uy;
+    const double uu15 = 1.5 * (ux * ux + uy * uy);
     double dudx = 0.0, dudy = 0.0, dvdx = 0.0, dvdy = 0.0;
     if (with_noneq) {
       dudx = diff1(u, p, x, y, 1, 0);
@@ -1143,18 +1146,41 @@ __global__ void init_device_kernel(S *__restrict__ A, StepParams p, const float 
       dvdx = diff1(v, p, x, y, 1, 0);
       dvdy = diff1(v, p, x, y, 0, 1);
     }
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      const double cu = CX(k) * ux + CY(k) * uy;
-      double f = WD(k) * r * (1.0 + 3.0 * cu + 4.5 * cu * cu - 1.5 * uu);
+    // Opposite directions share all but the sign of 3 cu, directions of one weight
+    // their factors; products with a zero component of c are left out.  Every
+    // operation that remains is the formula's, in its order.
+    auto put = [&](int k, double wr, double cu3, double cuu, double q) {
+      double f = wr * (1.0 + cu3 + cuu - uu15);
       if (with_noneq) {
         // stored state is post-collision: f*_neq = (1 - 1/tau) f_neq, and
         // (1 - 1/tau) (-tau w rho / c_s^2) = -(tau - 1) w rho / c_s^2
-        const double qxx = CX(k) * CX(k) - 1.0 / 3.0, qyy = CY(k) * CY(k) - 1.0 / 3.0, qxy = CX(k) * CY(k);
-        f -= 3.0 * (tau - 1.0) * WD(k) * r * (qxx * dudx + qyy * dvdy + qxy * (dudy + dvdx));
+        f -= q;
       }
-      A[(size_t)k * p.plane + o] = Store<S>::st((typename Store<S>::C)(f - ref_pop(k, p.U)));
+      A[(size_t)k * p.plane + o] = Store<S>::st((typename Store<S>::C)(f - rp[k]));
+    };
+    const double n3 = 3.0 * (tau - 1.0), shear = dudy + dvdx;
+    constexpr double qd = 1.0 - 1.0 / 3.0, q0 = 0.0 - 1.0 / 3.0;
+    double qx = 0.0, qy = 0.0, qp = 0.0, qm = 0.0, qr = 0.0;
+    if (with_noneq) {
+      const double na = n3 * WD(1) * r, nd = n3 * WD(5) * r, dd = qd * dudx + qd * dvdy;
+      qx = na * (qd * dudx + q0 * dvdy);
+      qy = na * (q0 * dudx + qd * dvdy);
+      qp = nd * (dd + shear);
+      qm = nd * (dd - shear);
+      qr = n3 * WD(0) * r * (q0 * dudx + q0 * dvdy);
     }
+    const double wa = WD(1) * r, wd = WD(5) * r, cp = ux + uy, cm = uy - ux;
+    put(0, WD(0) * r, 0.0, 0.0, qr);
+    const double x3 = 3.0 * ux, xx = 4.5 * ux * ux, y3 = 3.0 * uy, yy = 4.5 * uy * uy;
+    const double p3 = 3.0 * cp, pp = 4.5 * cp * cp, m3 = 3.0 * cm, mm = 4.5 * cm * cm;
+    put(1, wa, x3, xx, qx);
+    put(3, wa, -x3, xx, qx);
+    put(2, wa, y3, yy, qy);
+    put(4, wa, -y3, yy, qy);
+    put(5, wd, p3, pp, qp);
+    put(7, wd, -p3, pp, qp);
+    put(6, wd, m3, mm, qm);
+    put(8, wd, -m3, mm, qm);
   }
 }
 
@@ -1567,7 +1593,8 @@ struct Launch {
   static cudaError_t init_device(void *A, const StepParams &p, const float *r, const float *u, const float *v,
                                  int with_noneq, double tau, cudaStream_t st) {
     const long long n = (long long)p.nx * p.ny;
-    const int blocks = (int)((n + 255) / 256 < 65535 * 8 ? (n + 255) / 256 : 65535 * 8);
+    // a few nodes per thread: the reference populations are computed once
+    const int blocks = (int)((n + 255) / 256 < 152 * 16 ? (n + 255) / 256 : 152 * 16);
     init_device_kernel<S><<<blocks > 0 ? blocks : 1, 256, 0, st>>>((S *)A, p, r, u, v, with_noneq, tau);
     return cudaGetLastError();
   }
