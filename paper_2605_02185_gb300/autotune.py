@@ -2,7 +2,8 @@
 
 For a lattice (or a batch of lattices) it times every candidate shape of the
 step kernel -- the persistent bulk-copy kernel with (compute warps, nodes per
-thread, pipeline stages) and resident CTAs per SM, plus the direct kernel --
+thread, pipeline stages) and resident CTAs per SM, the direct kernel, and the
+library's own choice (two steps per pass for float storage) --
 with CUDA events on the context's stream, and keeps the fastest.  Results are
 cached as JSON per (GPU name, lattice sizes, storage type) so a later run
 picks the shape without timing again.
@@ -15,6 +16,7 @@ import json
 import os
 
 DIRECT = "direct"
+AUTO = "auto"
 
 
 def cache_path() -> str:
@@ -42,12 +44,12 @@ def _save(path, data):
 
 def cache_key(gpu_name: str, sizes, storage: int) -> str:
     sz = ",".join(f"{nx}x{ny}" for nx, ny in sizes)
-    return f"{gpu_name}|s{storage}|{sz}"
+    return f"{gpu_name}|s{storage}|{sz}|{AUTO}"  # the last part: what the candidates include
 
 
 def candidates(ctas=(1, 2)):
     from . import lbm
-    out = [(DIRECT, None, 1)]
+    out = [(AUTO, None, 0), (DIRECT, None, 1)]
     for shp in lbm.lbm_kernel_shapes():
         for c in ctas:
             out.append(("tma", shp, c))
@@ -62,7 +64,9 @@ def time_candidate(target, cand, steps: int, warmup: int, stream) -> float:
 
     kind, shape, ctas = cand
     try:
-        if kind == DIRECT:
+        if kind == AUTO:
+            target.set_kernel(lbm.LBM_KERNEL_AUTO)
+        elif kind == DIRECT:
             target.set_kernel(lbm.LBM_KERNEL_DIRECT)
         else:
             target.set_kernel(lbm.LBM_KERNEL_TMA, *shape, ctas_per_sm=ctas)
@@ -115,7 +119,9 @@ def tune(target, sizes, storage: int, stream, steps: int = 20, warmup: int = 4, 
         if use_cache:
             data[key] = best
             _save(path, data)
-    if best["kind"] == DIRECT:
+    if best["kind"] == AUTO:
+        target.set_kernel(lbm.LBM_KERNEL_AUTO)
+    elif best["kind"] == DIRECT:
         target.set_kernel(lbm.LBM_KERNEL_DIRECT)
     else:
         target.set_kernel(lbm.LBM_KERNEL_TMA, *best["shape"], ctas_per_sm=best["ctas_per_sm"])
