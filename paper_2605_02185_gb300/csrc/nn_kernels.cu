@@ -367,7 +367,16 @@ __global__ void __launch_bounds__(W9_THREADS) conv_wgrad9_kernel(const bf16 *__r
         atomicAdd(dst + 1, acc[mt][nt][2 * hf + 1]);
       }
     }
-  if (do_bias && o0 + lane < cout) atomicAdd(gb + o0 + lane, bsum);
+  if (do_bias) {  // one atomic per channel and block: each rounds against the whole sum
+    __shared__ float part[9][32];
+    part[warp][lane] = bsum;
+    __syncthreads();
+    if (warp == 0 && o0 + lane < cout) {
+      float s = 0.f;
+      for (int q = 0; q < 9; ++q) s += part[q][lane];
+      atomicAdd(gb + o0 + lane, s);
+    }
+  }
 }
 
 // wf[c, dy, dx, o] = w[o, 2-dy, 2-dx, c]
