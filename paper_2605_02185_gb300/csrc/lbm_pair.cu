@@ -20,7 +20,9 @@ struct Window {
 };
 
 // Cost of a row of the inlet's or outlet's window, and of a row that meets the
-// body, against a plain row.
+// body, against a plain row.  A pass ends with its slowest cell: 3200 x 1600 with
+// body rows counted as 1, 1.3, 1.6 and 2 plain ones ran at 61, 53, 47 and 45 us a
+// step, edge windows at 1.4 instead of 1.2 made no difference.
 constexpr double kEdgeCost = 1.2, kBodyCost = 2.0;
 
 // Nodes from which a launch runs one pass only.  Within a launch the cells drift
