@@ -24,6 +24,9 @@ struct Window {
 // body rows counted as 1, 1.3, 1.6 and 2 plain ones ran at 61, 53, 47 and 45 us a
 // step, edge windows at 1.4 instead of 1.2 made no difference.
 constexpr double kEdgeCost = 1.2, kBodyCost = 2.0;
+// Cost of a cell beyond its rows, in plain rows: two rows computed twice, the
+// filling of its ring.
+constexpr double kCellCost = 3.0;
 
 // Nodes from which a launch runs one pass only.  Within a launch the cells drift
 // apart, and on a large lattice the columns and DRAM pages that neighbouring
@@ -68,14 +71,29 @@ int pair_plan(const std::vector<PairLattice> &lattices, int sms, void *region, i
   auto bands = [&](const Window &v, double cost) {
     return std::max(1, std::min(lattices[v.lat].ny, (int)std::ceil(v.total / cost)));
   };
-  double lo = 1.0, hi = 1.0;
-  for (const Window &v : win) hi = std::max(hi, v.total);
-  for (int k = 0; k < 40; ++k) {
-    const double mid = 0.5 * (lo + hi);
-    long long n = 0;
-    for (const Window &v : win) n += bands(v, mid);
-    if (n <= warps) hi = mid;
-    else lo = mid;
+  double most = 1.0;
+  for (const Window &v : win) most = std::max(most, v.total);
+  auto cheapest = [&](int n_max) {  // the least cost per cell that needs at most n_max cells
+    double lo = 1.0, up = most;
+    for (int k = 0; k < 40; ++k) {
+      const double mid = 0.5 * (lo + up);
+      long long n = 0;
+      for (const Window &v : win) n += bands(v, mid);
+      if (n <= n_max) up = mid;
+      else lo = mid;
+    }
+    return up;
+  };
+  // Where few bands fit (wide lattices), a second or third cell per warp wastes
+  // fewer of the warps: 40000 x 3000 has 667 windows, so three bands leave a
+  // sixth of 2,432 warps idle and ran at 1324 us a step, seven at 964.
+  double hi = cheapest(warps);
+  for (int rounds = 2; rounds <= 3; ++rounds) {
+    const double c = cheapest(rounds * warps);
+    if (rounds * (c + kCellCost) < 0.95 * (hi + kCellCost) && (long long)rounds * warps <= cells_cap) {
+      hi = c;
+      break;
+    }
   }
   std::vector<int4> cells;
   std::vector<double> place;  // a cell's height in its lattice

@@ -13,7 +13,7 @@ namespace gblbm {
 
 // Capacities of a workspace region for `cases` lattices; a plan that needs more
 // leaves its lattices to the one-step kernels.
-constexpr int kPairCellsSingle = 4096, kPairSlotsSingle = 512;
+constexpr int kPairCellsSingle = 8192, kPairSlotsSingle = 512;
 constexpr int kPairCellsBatch = 8192, kPairSlotsBatch = 4096;
 size_t pair_region_bytes(int cells, int slots, int cases);
 
