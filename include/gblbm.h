@@ -185,7 +185,9 @@ int lbm_init_fields(lbm_ctx *ctx, const double *rho, const double *u, const doub
 int lbm_init_fields_device(lbm_ctx *ctx, const float *rho, const float *u, const float *v, int with_noneq);
 
 /* Advance n >= 0 steps (asynchronous on the context stream).  Step n maps
- * f*(n-1) to f*(n) and appends the force of f*(n) to the history. */
+ * f*(n-1) to f*(n) and appends the force of f*(n) to the history.  May be
+ * called while the caller captures the stream: the graph of an even number of
+ * steps ends in the buffer it begins in and can be launched repeatedly. */
 int lbm_step(lbm_ctx *ctx, int64_t n);
 
 /* Wait for the context stream; report LBM_ERR_UNSTABLE / LBM_ERR_TIMEOUT if

@@ -484,9 +484,10 @@ int lbm_step(lbm_ctx *c, int64_t n) {
   CK(cudaSetDevice(c->dev));
   if (c->kernel == LBM_KERNEL_TMA_WAVE) return wave_steps(c, n);
   if (c->pair) {
-    const int rc = pair_steps(c, n & ~(int64_t)1);
+    const int64_t m = pair_steps_of(c->stream, n);
+    const int rc = pair_steps(c, m);
     if (rc) return rc;
-    n &= 1;
+    n -= m;
   }
   while (n > 0) {
     if (c->graph && c->cur == 0 && n >= c->graph_steps) {

@@ -310,9 +310,10 @@ int lbm_batch_step(lbm_batch *b, int64_t n) {
     if (!c->inited) return LBM_ERR_STATE;
   CK(cudaSetDevice(b->dev));
   if (b->pair) {
-    const int rc = batch_pair_steps(b, n & ~(int64_t)1);
+    const int64_t m = pair_steps_of(b->stream, n);
+    const int rc = batch_pair_steps(b, m);
     if (rc) return rc;
-    n &= 1;
+    n -= m;
   }
   while (n > 0) {
     if (b->graph && b->cur == 0 && n >= b->graph_steps) {

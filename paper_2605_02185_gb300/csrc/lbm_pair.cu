@@ -191,6 +191,13 @@ int pair_plan(const std::vector<PairLattice> &lattices, int sms, void *region, i
   return LBM_OK;
 }
 
+int64_t pair_steps_of(cudaStream_t st, int64_t n) {
+  if (n < 2) return 0;
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &status) != cudaSuccess) cudaGetLastError();  // the launch reports it
+  return n & ~(int64_t)(status == cudaStreamCaptureStatusNone ? 1 : 3);
+}
+
 cudaError_t pair_reset(const PairParams &q, cudaStream_t st) {
   return cudaMemsetAsync(q.flags, 0, (size_t)q.ncells * sizeof(unsigned), st);
 }

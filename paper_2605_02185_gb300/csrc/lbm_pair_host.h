@@ -4,6 +4,7 @@
 
 #include <cuda_runtime.h>
 
+#include <cstdint>
 #include <vector>
 
 #include "lbm_ctx.h"
@@ -28,6 +29,10 @@ struct PairLattice {
 // where the kernel does not take them.
 int pair_plan(const std::vector<PairLattice> &lattices, int sms, void *region, int cells_cap, int slots_cap,
               cudaStream_t st, PairParams *q, int *grid);
+// Of n steps, those to take in pairs: all but an odd one.  Under a caller's stream
+// capture a multiple of four, so that an even number of steps ends in the buffer it
+// began in (each pass changes it) and the graph can be launched again.
+int64_t pair_steps_of(cudaStream_t st, int64_t n);
 // Clear the cells' flags (a new state; a launch that gave up left them uneven).
 cudaError_t pair_reset(const PairParams &q, cudaStream_t st);
 
