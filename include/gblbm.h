@@ -283,7 +283,10 @@ int lbm_kernel_shapes_for(int kernel, int *out, int cap, int *count);
  * path testable: the waits give up after wait_seconds (<= 0: the default
  * 1 s; at most 60), and if tile >= 0 the TMA producer announces the copies
  * of row tile `tile` (row * tiles per row + segment, as the kernel numbers
- * them) but never issues them, so the waits on that tile run out.  The
+ * them) but never issues them, so the waits on that tile run out.  Where two
+ * steps at a time run in one pass, the warps of that row do not report their
+ * passes, so their neighbours' waits run out (a call of fewer than four steps
+ * then takes the one-step kernel, as one pass waits for nothing).  The
  * populations are then partly stale: restore a checkpoint or re-initialise.
  * The context must use LBM_KERNEL_TMA, LBM_KERNEL_TMA_BULK or
  * LBM_KERNEL_TMA_WAVE (LBM_ERR_ARG otherwise).  tile < 0 and wait_seconds <= 0 restore normal operation. */
@@ -365,6 +368,9 @@ int lbm_batch_sync(lbm_batch *batch);
 int lbm_batch_set_kernel(lbm_batch *batch, int kernel, int consumer_warps, int cells_per_thread, int stages,
                          int ctas_per_sm);
 int lbm_batch_get_kernel(lbm_batch *batch, int *out6);
+/* lbm_set_fault_injection for a batch on LBM_KERNEL_TMA (LBM_ERR_ARG
+ * otherwise): row tile `tile` of case c; the wait limit holds for every case. */
+int lbm_batch_set_fault_injection(lbm_batch *batch, int c, int64_t tile, double wait_seconds);
 int lbm_batch_get_stream(lbm_batch *batch, void **stream);
 int lbm_batch_launch_count(lbm_batch *batch, int64_t *count);
 /* Total nodes of all cases, and the algorithmic HBM bytes of one batch step. */

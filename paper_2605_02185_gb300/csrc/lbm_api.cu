@@ -169,7 +169,6 @@ int configure_kernel(lbm_ctx *c, int kernel, int shape, int ctas_per_sm) {
 // (LBM_KERNEL_AUTO, no explicit shape).
 int configure_pair(lbm_ctx *c, bool automatic) {
   c->pair = false;
-  c->pair_auto = automatic;
   c->pair_grid = 0;
   if (!automatic || c->o.storage != LBM_F32 || c->kernel != LBM_KERNEL_TMA) return LBM_OK;
   CK(pair_f32(0, nullptr, nullptr, c->p, c->pq, nullptr, 1, nullptr));
@@ -189,6 +188,10 @@ int pair_steps(lbm_ctx *c, int64_t n) {
   while (n > 0) {
     PairParams q = c->pq;
     q.pairs = (int)std::min<int64_t>(n / 2, c->pq.pairs);
+    if (c->p.fault_tile >= 0) {
+      q.fault_case = 0;
+      q.fault_row = c->p.fault_tile / c->nseg;
+    }
     CK(pair_f32(c->pair_grid, c->buf[c->cur], c->buf[c->cur ^ 1], c->p, q, c->stream, 0, nullptr));
     c->cur ^= q.pairs & 1;
     c->launches += 2;
@@ -483,7 +486,7 @@ int lbm_step(lbm_ctx *c, int64_t n) {
   if (!c->inited) return LBM_ERR_STATE;
   CK(cudaSetDevice(c->dev));
   if (c->kernel == LBM_KERNEL_TMA_WAVE) return wave_steps(c, n);
-  if (c->pair) {
+  if (c->pair && pair_waits(c->p, c->pq, n)) {
     const int64_t m = pair_steps_of(c->stream, n);
     const int rc = pair_steps(c, m);
     if (rc) return rc;
@@ -662,7 +665,6 @@ int lbm_set_fault_injection(lbm_ctx *c, int64_t tile, double wait_seconds) {
   if (tile >= (int64_t)c->ny * c->nseg || !(wait_seconds <= 60.0)) return LBM_ERR_ARG;
   CK(cudaSetDevice(c->dev));
   CK(cudaStreamSynchronize(c->stream));
-  c->pair = c->pair_grid > 0 && c->pair_auto && tile < 0 && !(wait_seconds > 0);  // the injection is the one-step kernel's
   c->p.fault_tile = tile < 0 ? -1 : (int)tile;
   c->p.wait_ns = wait_seconds > 0 ? (unsigned long long)(wait_seconds * 1e9) : 1000000000ull;
   if (c->p.wait_ns == 0) c->p.wait_ns = 1;

@@ -45,6 +45,7 @@ struct lbm_batch {
   int pair_grid = 0;
   PairParams pq{};
   void *pair_region = nullptr;
+  int fault_case = -1;  // the case a fault is injected into
 };
 
 namespace {
@@ -83,18 +84,8 @@ int batch_sizes(int n, const lbm_case *cases, const lbm_opts *common, std::vecto
   return LBM_OK;
 }
 
-// Give every case the tile width of the batch kernel, then upload the
-// per-case descriptors with the batch-wide tile offsets.
-int configure_batch(lbm_batch *b, int kernel, int shape, int ctas) {
-  if (kernel == LBM_KERNEL_TMA_BULK) return LBM_ERR_ARG;  // single-lattice kernel only
-  const TmaShape &ts = kTmaShapes[shape];
-  for (lbm_ctx *c : b->cases) {
-    const int rc = kernel == LBM_KERNEL_DIRECT ? lbm_set_kernel(c, LBM_KERNEL_DIRECT, 0, 0, 0, 1)
-                                               : lbm_set_kernel(c, LBM_KERNEL_TMA, ts.ncw, ts.cpt, ts.stages, ctas);
-    if (rc) return rc;
-  }
-  const KernelOps *ops = b->cases[0]->ops;
-  if (kernel != LBM_KERNEL_DIRECT) CK(ops->batch_prep(shape));
+// Upload the per-case descriptors with the batch-wide tile offsets.
+int upload_desc(lbm_batch *b) {
   std::vector<CaseDesc> h(b->cases.size());
   long long item0 = 0, nodes = 0;
   for (size_t i = 0; i < b->cases.size(); ++i) {
@@ -111,10 +102,26 @@ int configure_batch(lbm_batch *b, int kernel, int shape, int ctas) {
   CK(cudaStreamSynchronize(b->stream));
   b->nitems = item0;
   b->nodes = nodes;
+  return LBM_OK;
+}
+
+// Give every case the tile width of the batch kernel and upload the descriptors.
+int configure_batch(lbm_batch *b, int kernel, int shape, int ctas) {
+  if (kernel == LBM_KERNEL_TMA_BULK) return LBM_ERR_ARG;  // single-lattice kernel only
+  const TmaShape &ts = kTmaShapes[shape];
+  for (lbm_ctx *c : b->cases) {
+    const int rc = kernel == LBM_KERNEL_DIRECT ? lbm_set_kernel(c, LBM_KERNEL_DIRECT, 0, 0, 0, 1)
+                                               : lbm_set_kernel(c, LBM_KERNEL_TMA, ts.ncw, ts.cpt, ts.stages, ctas);
+    if (rc) return rc;
+  }
+  const KernelOps *ops = b->cases[0]->ops;
+  if (kernel != LBM_KERNEL_DIRECT) CK(ops->batch_prep(shape));
   b->kernel = kernel;
   b->shape = shape;
+  const int rc = upload_desc(b);
+  if (rc) return rc;
   b->ctas = kernel == LBM_KERNEL_DIRECT ? 0 : b->cases[0]->ctas_per_sm;
-  b->grid = kernel == LBM_KERNEL_DIRECT ? (int)item0 : (int)std::min<long long>(item0, (long long)b->sms * b->ctas);
+  b->grid = kernel == LBM_KERNEL_DIRECT ? (int)b->nitems : (int)std::min<long long>(b->nitems, (long long)b->sms * b->ctas);
   return LBM_OK;
 }
 
@@ -143,6 +150,11 @@ int batch_pair_steps(lbm_batch *b, int64_t n) {
     PairParams q = b->pq;
     q.pairs = (int)std::min<int64_t>(n / 2, b->pq.pairs);
     q.parity = b->cur;
+    if (b->fault_case >= 0) {
+      const lbm_ctx *f = b->cases[b->fault_case];
+      q.fault_case = b->fault_case;
+      q.fault_row = f->p.fault_tile / f->nseg;
+    }
     CK(pair_batch_f32(b->pair_grid, b->desc, (int)b->cases.size(), mrt, q, b->stream, 0, nullptr));
     b->cur ^= q.pairs & 1;
     b->launches += 2;
@@ -309,7 +321,7 @@ int lbm_batch_step(lbm_batch *b, int64_t n) {
   for (lbm_ctx *c : b->cases)
     if (!c->inited) return LBM_ERR_STATE;
   CK(cudaSetDevice(b->dev));
-  if (b->pair) {
+  if (b->pair && (b->fault_case < 0 || pair_waits(b->cases[b->fault_case]->p, b->pq, n))) {
     const int64_t m = pair_steps_of(b->stream, n);
     const int rc = batch_pair_steps(b, m);
     if (rc) return rc;
@@ -362,6 +374,17 @@ int lbm_batch_set_kernel(lbm_batch *b, int kernel, int ncw, int cpt, int stages,
   rc = configure_batch_pair(b, automatic);
   if (rc) return rc;
   return capture_batch_graph(b);
+}
+
+int lbm_batch_set_fault_injection(lbm_batch *b, int c, int64_t tile, double wait_seconds) {
+  if (!valid_case(b, c) || b->kernel != LBM_KERNEL_TMA) return LBM_ERR_ARG;
+  if (tile >= (int64_t)b->cases[c]->ny * b->cases[c]->nseg || !(wait_seconds <= 60.0)) return LBM_ERR_ARG;
+  for (int i = 0; i < (int)b->cases.size(); ++i) {
+    const int rc = lbm_set_fault_injection(b->cases[i], i == c ? tile : -1, wait_seconds);
+    if (rc) return rc;
+  }
+  b->fault_case = tile < 0 ? -1 : c;
+  return upload_desc(b);
 }
 
 int lbm_batch_get_kernel(lbm_batch *b, int *out6) {

@@ -57,7 +57,7 @@ struct lbm_ctx {
   int kernel = LBM_KERNEL_TMA, shape = 0, ctas_per_sm = 1, grid = 0, seg = 0, nseg = 0;
   gblbm::StepParams p{};
   // two-step kernel: in use, its grid, the split of the lattice, their memory
-  bool pair = false, pair_auto = false;
+  bool pair = false;
   int pair_grid = 0;
   gblbm::PairParams pq{};
   void *pair_region = nullptr;

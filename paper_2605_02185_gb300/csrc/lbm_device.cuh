@@ -819,6 +819,7 @@ struct PairParams {
   const int2 *case_slots;   // batch: slots [x, y) of each case
   int ncells, nslots;
   int pairs, parity;        // passes of this launch (on the host: at most); batch: the buffer it starts from
+  int fault_case, fault_row;  // failure-path test: the cells of this row of this lattice report no pass (-1: none)
 };
 
 // ---- multi-step kernel: per-row completion counters ------------------------

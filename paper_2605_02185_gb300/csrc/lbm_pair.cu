@@ -182,6 +182,7 @@ int pair_plan(const std::vector<PairLattice> &lattices, int sms, void *region, i
   q->nslots = slots;
   q->pairs = nodes < kPairManyNodes ? kPairMax : 1;
   q->parity = 0;
+  q->fault_case = q->fault_row = -1;
   CK(cudaMemcpyAsync(d_cells, cells.data(), cells.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(d_deps, deps.data(), deps.size() * sizeof(int), cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(d_ranges, ranges.data(), ranges.size() * sizeof(int2), cudaMemcpyHostToDevice, st));

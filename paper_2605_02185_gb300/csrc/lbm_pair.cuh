@@ -468,7 +468,7 @@ __global__ void __launch_bounds__(NW * 32, 1)
     // the pass is done: this cell's nodes are written, its neighbours' are read
     cp_async_wait<0>();
     __syncwarp();
-    if (lane == 0) {
+    if (lane == 0 && !(cd.x >> 16 == q.fault_case && a <= q.fault_row && q.fault_row < b)) {
       fence_acq_rel_gpu();
       st_relaxed_gpu(q.flags + cell, base_pass + (unsigned)pass + 1u);
     }

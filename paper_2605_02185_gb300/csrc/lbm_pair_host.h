@@ -33,6 +33,12 @@ int pair_plan(const std::vector<PairLattice> &lattices, int sms, void *region, i
 // capture a multiple of four, so that an even number of steps ends in the buffer it
 // began in (each pass changes it) and the graph can be launched again.
 int64_t pair_steps_of(cudaStream_t st, int64_t n);
+// False where a fault is injected but no cell of these n steps would wait for another
+// (a launch of one pass): the one-step kernel, whose tiles wait for their copies, then
+// takes them.
+inline bool pair_waits(const StepParams &p, const PairParams &q, int64_t n) {
+  return p.fault_tile < 0 || (n >= 4 && q.pairs >= 2);
+}
 // Clear the cells' flags (a new state; a launch that gave up left them uneven).
 cudaError_t pair_reset(const PairParams &q, cudaStream_t st);
 

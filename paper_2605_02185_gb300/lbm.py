@@ -123,6 +123,7 @@ def load_library(path: str | None = None):
         "lbm_batch_step": (i, [vp, i64]),
         "lbm_batch_sync": (i, [vp]),
         "lbm_batch_set_kernel": (i, [vp, i, i, i, i, i]),
+        "lbm_batch_set_fault_injection": (i, [vp, i, i64, d]),
         "lbm_batch_get_kernel": (i, [vp, vp]),
         "lbm_batch_get_stream": (i, [vp, ctypes.POINTER(vp)]),
         "lbm_batch_launch_count": (i, [vp, ctypes.POINTER(i64)]),
@@ -564,6 +565,12 @@ def lbm_batch_sync(h):
 def lbm_batch_set_kernel(h, kernel: int, consumer_warps=0, cells_per_thread=0, stages=0, ctas_per_sm=0):
     _check(load_library().lbm_batch_set_kernel(h, int(kernel), int(consumer_warps), int(cells_per_thread),
                                                int(stages), int(ctas_per_sm)), "lbm_batch_set_kernel")
+
+
+def lbm_batch_set_fault_injection(h, c: int, tile: int, wait_seconds: float):
+    """lbm_set_fault_injection for row tile ``tile`` of case ``c`` (see gblbm.h)."""
+    _check(load_library().lbm_batch_set_fault_injection(h, int(c), int(tile), float(wait_seconds)),
+           "lbm_batch_set_fault_injection")
 
 
 def lbm_batch_get_kernel(h) -> dict:
