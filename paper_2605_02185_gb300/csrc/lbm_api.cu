@@ -209,14 +209,10 @@ cudaError_t launch_step(lbm_ctx *c, int from) {
   return c->ops->tma(c->shape, c->grid, A, B, c->p, c->stream);
 }
 
-// Clear the multi-step kernels' counters (a new state, or the recovery
+// Clear the multi-step kernel's row counters (a new state, or the recovery
 // from a launch that gave up and left them uneven).
 cudaError_t reset_wave_rows(lbm_ctx *c) {
   c->wave_base = 0;
-  if (c->pair) {
-    const cudaError_t e = pair_reset(c->pq, c->stream);
-    if (e != cudaSuccess) return e;
-  }
   return cudaMemsetAsync(c->wave_rows, 0, (size_t)c->ny * sizeof(unsigned), c->stream);
 }
 

@@ -306,7 +306,6 @@ int lbm_batch_init_fields(lbm_batch *b, int c, const double *rho, const double *
   // the batch steps all cases with one parity: bring this case's f*(0) to it
   int rc = lbm_init_fields(ctx, rho, u, v);
   if (rc) return rc;
-  if (b->pair) CK(pair_reset(b->pq, b->stream));
   if (b->cur != 0) {
     CK(cudaMemcpyAsync(ctx->buf[1], ctx->buf[0], (size_t)9 * ctx->plane * ctx->elem, cudaMemcpyDeviceToDevice,
                        b->stream));

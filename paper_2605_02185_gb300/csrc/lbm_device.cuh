@@ -814,7 +814,7 @@ __device__ __forceinline__ void named_bar(int id, int threads) {
 struct PairParams {
   const int4 *cells;        // (case << 16 | window, first row, past the last row, force slot or -1)
   const int *deps;          // [ncells][32] the cells a cell exchanges nodes with, then -1
-  unsigned *flags;          // [ncells] passes done since the flags were last cleared
+  unsigned *flags;          // [ncells] passes done in this launch; zero between launches
   double2 *slots;           // [2 pairs][nslots] force partials of the cells that own links
   const int2 *case_slots;   // batch: slots [x, y) of each case
   int ncells, nslots;

@@ -199,8 +199,4 @@ int64_t pair_steps_of(cudaStream_t st, int64_t n) {
   return n & ~(int64_t)(status == cudaStreamCaptureStatusNone ? 1 : 3);
 }
 
-cudaError_t pair_reset(const PairParams &q, cudaStream_t st) {
-  return cudaMemsetAsync(q.flags, 0, (size_t)q.ncells * sizeof(unsigned), st);
-}
-
 }  // namespace gblbm

@@ -117,11 +117,13 @@ __device__ __forceinline__ void pair_wall(int bc, bool bottom, float U, float (&
 }
 
 // History entries of a launch: block c its case c, one warp per step, each
-// step's slots of the case summed in slot order.
+// step's slots of the case summed in slot order.  Clears the cells' flags for the
+// next launch, whatever this one left of them (one that gave up leaves them uneven).
 static __global__ void __launch_bounds__(1024) pair_finish(StepParams p0, const CaseDesc *cases, PairParams q) {
   const StepParams &p = cases ? cases[blockIdx.x].p : p0;
   const int2 range = q.case_slots ? q.case_slots[blockIdx.x] : make_int2(0, q.nslots);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < q.ncells; i += gridDim.x * blockDim.x) q.flags[i] = 0;
   const unsigned long long n0 = *p.step;
   for (int s = warp; s < 2 * q.pairs; s += 32) {
     double sx, sy;
@@ -152,7 +154,6 @@ __global__ void __launch_bounds__(NW * 32, 1)
   if (first >= q.ncells) return;
   const StepParams &p = BATCH ? sp[warp] : p0;
   float *tiles = reinterpret_cast<float *>(smem + warp * Lay::WARP);
-  const unsigned base_pass = ld_relaxed_gpu(q.flags + first);  // every cell stands at the same count
 
 #pragma unroll 1
   for (int pass = 0; pass < q.pairs; ++pass)
@@ -178,12 +179,12 @@ __global__ void __launch_bounds__(NW * 32, 1)
     }
     if (pass > 0) {  // the neighbours' last pass
       const int dep = __ldg(q.deps + (size_t)cell * 32 + lane);
-      const unsigned need = base_pass + (unsigned)pass;
-      bool ok = dep < 0 || (int)(ld_relaxed_gpu(q.flags + max(dep, 0)) - need) >= 0;
+      const unsigned need = (unsigned)pass;
+      bool ok = dep < 0 || ld_relaxed_gpu(q.flags + max(dep, 0)) >= need;
       if (!__all_sync(0xffffffffu, ok)) {
         const unsigned long long t0 = global_ns(), lim = wait_limit(p.wait_ns);
         while (true) {
-          if (!ok) ok = (int)(ld_relaxed_gpu(q.flags + dep) - need) >= 0;
+          if (!ok) ok = ld_relaxed_gpu(q.flags + dep) >= need;
           if (__all_sync(0xffffffffu, ok)) break;
           if (__any_sync(0xffffffffu, global_ns() - t0 > lim)) {
             if (lane == 0) atomicOr(p.err, ERR_TIMEOUT);
@@ -470,7 +471,7 @@ __global__ void __launch_bounds__(NW * 32, 1)
     __syncwarp();
     if (lane == 0 && !(cd.x >> 16 == q.fault_case && a <= q.fault_row && q.fault_row < b)) {
       fence_acq_rel_gpu();
-      st_relaxed_gpu(q.flags + cell, base_pass + (unsigned)pass + 1u);
+      st_relaxed_gpu(q.flags + cell, (unsigned)pass + 1u);
     }
   }
 }

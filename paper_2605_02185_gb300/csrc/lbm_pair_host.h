@@ -39,7 +39,5 @@ int64_t pair_steps_of(cudaStream_t st, int64_t n);
 inline bool pair_waits(const StepParams &p, const PairParams &q, int64_t n) {
   return p.fault_tile < 0 || (n >= 4 && q.pairs >= 2);
 }
-// Clear the cells' flags (a new state; a launch that gave up left them uneven).
-cudaError_t pair_reset(const PairParams &q, cudaStream_t st);
 
 }  // namespace gblbm

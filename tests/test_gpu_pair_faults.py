@@ -41,7 +41,7 @@ def same(got, want):
 
 
 # 2 steps: one pass, which waits for nothing, so the one-step kernel takes them
-@pytest.mark.parametrize("steps", [2, 4, 64])
+@pytest.mark.parametrize("steps", [2, 4, 64, 70])
 @pytest.mark.parametrize("bounce", [lbm.LBM_BOUNCE_HALFWAY, lbm.LBM_BOUNCE_INTERPOLATED], ids=["half", "interp"])
 @pytest.mark.parametrize("size,bc", [((301, 57), W.BC_FREESLIP), ((61, 30), W.BC_PERIODIC), ((800, 400), W.BC_ZOUHE)],
                          ids=["301x57", "61x30", "800x400"])
@@ -90,7 +90,7 @@ def test_choosing_the_kernel_again_keeps_the_fault():
         lat.close()
 
 
-@pytest.mark.parametrize("steps", [2, 64])
+@pytest.mark.parametrize("steps", [2, 64, 70])
 def test_batch_times_out_and_recovers(steps):
     cases = [W.random_case(97, 33, 1, W.BC_FREESLIP, D=8), W.random_case(241, 59, 4, W.BC_MOVINGWALL, D=10),
              W.random_case(400, 120, 3, W.BC_ZOUHE, D=20)]
@@ -106,6 +106,49 @@ def test_batch_times_out_and_recovers(steps):
         b.sync()
         for c, wl in enumerate(cases):
             same((b.get_populations(c), b.forces_raw(c)), direct(wl, 70))
+    finally:
+        b.close()
+
+
+def test_recovery_past_other_kernels():
+    # timed out, then a new state while the library's choice does not run, and back
+    wl = W.random_case(301, 57, seed=5, bc=W.BC_FREESLIP, D=8)
+    lat = lbm.lattice_for(wl)
+    try:
+        lat.init_fields(*wl.initial_fields())
+        start = lat.get_populations()
+        lbm.lbm_set_fault_injection(lat.h, 7, WAIT)
+        lat.step(70)
+        assert times_out(lat)
+        lbm.lbm_set_fault_injection(lat.h, -1, WAIT)
+        lat.set_populations(start, 1)
+        lat.step(1)
+        lbm.lbm_set_fault_injection(lat.h, -1, 0.0)
+        lat.step(69)
+        lat.sync()
+        want = direct(wl, 70)
+        same((lat.get_populations(), lat.forces_raw(1)), (want[0], want[1][1:]))
+    finally:
+        lat.close()
+
+
+def test_batch_recovery_through_its_cases():
+    cases = [W.random_case(97, 33, 1, W.BC_FREESLIP, D=8), W.random_case(241, 59, 4, W.BC_MOVINGWALL, D=10)]
+    b = lbm.Batch(cases)
+    try:
+        b.init_all()
+        starts = [b.get_populations(c) for c in range(2)]
+        lbm.lbm_batch_set_fault_injection(b.h, 0, 5, WAIT)
+        b.step(64)  # 32 passes: the batch stays on the buffer it began in
+        assert times_out(b)
+        lbm.lbm_batch_set_fault_injection(b.h, 0, -1, 0.0)
+        for c in range(2):
+            lbm.lbm_set_populations(b.case(c), starts[c], 1)
+        b.step(70)
+        b.sync()
+        for c, wl in enumerate(cases):
+            want = direct(wl, 70)
+            same((b.get_populations(c), b.forces_raw(c, 1)), (want[0], want[1][1:]))
     finally:
         b.close()
 
