@@ -502,6 +502,62 @@ __device__ __forceinline__ LF2 operator-(LF2 a, LF2 b) { return {__ffma2_rn(b.v,
 __device__ __forceinline__ LF2 operator*(LF2 a, LF2 b) { return {__fmul2_rn(a.v, b.v)}; }
 __device__ __forceinline__ LF2 fma(LF2 a, LF2 b, LF2 c) { return {__ffma2_rn(a.v, b.v, c.v)}; }
 
+// A sum of floats kept to three times their precision, 72 bits (two-sum, Knuth), so
+// that nothing a double sum holds is lost: this chip does about two double operations
+// per clock and SM, sixty times fewer than float ones.  Infinities, NaN and sums past
+// the float range do not survive it (infinity minus infinity appears in it): a caller
+// looks at hi.
+template <class L>
+__device__ __forceinline__ L two_sum(L a, L b, L &e) {
+  const L t = a + b, z = t - a;
+  e = (a - (t - z)) + (b - z);
+  return t;
+}
+template <class L>
+__device__ __forceinline__ L two_diff(L a, L b, L &e) {
+  const L t = a - b, z = t - a;
+  e = (a - (t - z)) - (b + z);
+  return t;
+}
+template <class L>
+struct Sum3 {
+  L hi{}, lo{}, rest{};
+  __device__ __forceinline__ void carry(L e) {
+    lo = two_sum(lo, e, e);
+    rest = rest + e;
+  }
+  __device__ __forceinline__ void add(L v) {
+    L e;
+    hi = two_sum(hi, v, e);
+    carry(e);
+  }
+  // |v| <= |hi| (Dekker's three operations)
+  __device__ __forceinline__ void add_smaller(L v) {
+    const L t = hi + v;
+    const L e = v - (t - hi);
+    hi = t;
+    carry(e);
+  }
+  // plus or minus the exact pair h + l
+  __device__ __forceinline__ void add(L h, L l) {
+    add(h);
+    carry(l);
+  }
+  __device__ __forceinline__ void sub(L h, L l) {
+    L e;
+    hi = two_diff(hi, h, e);
+    carry(e);
+    lo = two_diff(lo, l, e);
+    rest = rest + e;
+  }
+  // hi becomes the sum in float, lo the rest of it
+  __device__ __forceinline__ void normalize() {
+    L e;
+    hi = two_sum(hi, lo, e);
+    lo = e + rest;
+  }
+};
+
 // Negated reciprocal -1/x of a density (close to 1).  Float lanes: the
 // hardware estimate y of -1/x refined by one Newton-Raphson step,
 // e = 1 + x y, y' = y + y e, whose error is below one ulp; the refinement

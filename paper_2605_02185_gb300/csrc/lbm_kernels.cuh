@@ -1221,6 +1221,16 @@ __global__ void __launch_bounds__(256) force_kernel(const S *__restrict__ A, Ste
 }
 
 // ---- moments (Eq. 4) of the stored f* for rows [y0, y0 + rows) ---------
+__device__ __forceinline__ void node_moments(const double (&g)[9], double U, double &rho, double &u, double &v) {
+  const double drho = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
+  const double r = 1.0 + drho;
+  const double jx = U + ((g[1] - g[3]) + (g[5] - g[6]) + (g[8] - g[7]));
+  const double jy = (g[2] - g[4]) + (g[5] - g[8]) + (g[6] - g[7]);
+  rho = r;
+  u = jx / r;
+  v = jy / r;
+}
+
 template <class S, class O>
 __global__ void fields_kernel(const S *__restrict__ A, StepParams p, O *__restrict__ rho, O *__restrict__ u,
                               O *__restrict__ v, int y0, int rows) {
@@ -1235,24 +1245,35 @@ __global__ void fields_kernel(const S *__restrict__ A, StepParams p, O *__restri
       continue;
     }
     const size_t o = (size_t)y * p.pitch + x;
-    double g[9];
+    double g[9], m[3];
 #pragma unroll
     for (int k = 0; k < 9; ++k) g[k] = (double)Store<S>::ld(A[(size_t)k * p.plane + o]);
-    const double drho = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
-    const double r = 1.0 + drho;
-    const double jx = p.U + ((g[1] - g[3]) + (g[5] - g[6]) + (g[8] - g[7]));
-    const double jy = (g[2] - g[4]) + (g[5] - g[8]) + (g[6] - g[7]);
-    rho[i] = (O)r;
-    u[i] = (O)(jx / r);
-    v[i] = (O)(jy / r);
+    node_moments(g, p.U, m[0], m[1], m[2]);
+    rho[i] = (O)m[0];
+    u[i] = (O)m[1];
+    v[i] = (O)m[2];
   }
 }
 
-// The same for float output of float, half or bfloat16 storage, in float pairs
-// (about 48 bits) instead of double: on 16000 x 8000 the double form was bound
-// by its ~50 double operations a node (11.26 ms), this one reads 36 and writes
-// 12 bytes a node at the copy bandwidth.  N adjacent nodes per thread: 4 (16-byte
-// accesses) where nx and the output pointers allow it, else 1.
+// The same rounded to float (a function of its own: inlined in the kernel below, its
+// registers cost warps in flight).
+static __device__ __noinline__ float3 double_moments(float g0, float g1, float g2, float g3, float g4, float g5, float g6,
+                                                     float g7, float g8, double U) {
+  const double g[9] = {g0, g1, g2, g3, g4, g5, g6, g7, g8};
+  double r, u, v;
+  node_moments(g, U, r, u, v);
+  return make_float3((float)r, (float)u, (float)v);
+}
+
+// The moments of float, half or bfloat16 storage in float, summed in triples of floats (72
+// bits, where a double has 53) instead of double: on 16000 x 8000 the double form was
+// bound by its ~50 double operations a node (11.26 ms); this one takes 1.17 ms (bfloat16
+// 1.10), of which reading 36 and writing 12 bytes a node at the copy bandwidth is 0.92.
+// Pairs of floats took 0.89 ms, but left velocities near zero with wrong digits: their
+// 48 bits are too few where the terms cancel.
+// A node outside the range in which the triples hold (infinities, NaN, an offset above
+// 3/32, a velocity below 2^-100) takes the double form.  N adjacent nodes per thread: 4
+// (16-byte accesses) where nx and the output pointers allow it, else 1.
 template <class S, int N>
 __global__ void __launch_bounds__(256) fields_float_kernel(const S *__restrict__ A, const __grid_constant__ StepParams p,
                                                            float *__restrict__ rho, float *__restrict__ u,
@@ -1262,41 +1283,83 @@ __global__ void __launch_bounds__(256) fields_float_kernel(const S *__restrict__
   const unsigned per_row = (unsigned)p.nx / N, row = i / per_row;
   const int x = (int)(i - row * per_row) * N, y = y0 + (int)row;
   const S *src = A + (size_t)y * p.pitch + x;
-  float g[9][N];
+  float f[9][N];
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
     struct alignas(sizeof(S) * N) Pack { S s[N]; };
     const Pack t = *reinterpret_cast<const Pack *>(src + (size_t)k * p.plane);
 #pragma unroll
-    for (int j = 0; j < N; ++j) g[k][j] = (float)Store<S>::ld(t.s[j]);
+    for (int j = 0; j < N; ++j) f[k][j] = (float)Store<S>::ld(t.s[j]);
   }
-  const float Uh = (float)p.U, Ul = (float)(p.U - (double)Uh);
+  const float Uh = (float)p.U, Ul = (float)(p.U - (double)Uh), Ur = (float)(p.U - (double)Uh - (double)Ul);
   struct alignas(4 * N) Out { float s[N]; } o[3];
+  using L = typename std::conditional<N == 1, LF, LF2>::type;  // nodes in pairs
+  constexpr int LN = N == 1 ? 1 : 2;
+  auto both = [](float a) {
+    if constexpr (N == 1) return L{a};
+    else return L{make_float2(a, a)};
+  };
 #pragma unroll
-  for (int j = 0; j < N; ++j) {
-    Sum2 r, jx, jy;
-    r.hi = 1.f;
+  for (int j0 = 0; j0 < N; j0 += LN) {
+    L g[9];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) r.add(g[k][j]);
-    r.normalize();
-    jx.hi = Uh;
-    jx.lo = Ul;
-#pragma unroll
-    for (int k = 1; k < 9; ++k) {
-      if (CX(k)) jx.add(CX(k) > 0 ? g[k][j] : -g[k][j]);
-      if (CY(k)) jy.add(CY(k) > 0 ? g[k][j] : -g[k][j]);
+    for (int k = 0; k < 9; ++k) {
+      if constexpr (N == 1) g[k].v = f[k][j0];
+      else g[k].v = make_float2(f[k][j0], f[k][j0 + 1]);
     }
-    // quotient: an estimate and its remainder, rounded once
-    const float inv = rcp_estimate(r.hi);
-    auto div = [&](const Sum2 &a) {
-      const float q = __fmul_rn(a.hi, inv);
-      const float rem = __fadd_rn(__fmaf_rn(-q, r.hi, a.hi), __fmaf_rn(-q, r.lo, a.lo));
-      return __fmaf_rn(rem, inv, q);
-    };
-    const bool solid = (link_mask(p, x + j, y) & LM_SOLID) != 0;
-    o[0].s[j] = solid ? 1.f : r.hi;
-    o[1].s[j] = solid ? 0.f : div(jx);
-    o[2].s[j] = solid ? 0.f : div(jy);
+    Sum3<L> r, jx, jy;
+    r.hi = both(1.f);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) r.add_smaller(g[k]);  // 1 - 9 (3/32) > 3/32
+    L al, pl, ml;  // the exact differences both momenta are made of
+    const L ah = two_diff(g[1], g[3], al), ph = two_diff(g[5], g[7], pl), mh = two_diff(g[6], g[8], ml);
+    jx.hi = both(Uh);
+    jx.lo = both(Ul);
+    jx.rest = both(Ur);
+    jx.add(ah, al);
+    jx.add(ph, pl);
+    jx.sub(mh, ml);
+    jy.hi = two_diff(g[2], g[4], jy.lo);
+    jy.add(ph, pl);
+    jy.add(mh, ml);
+    r.normalize();
+    r.normalize();  // rho itself is an output: nearest also where lo lies at a tie
+    jx.normalize();
+    jy.normalize();
+#pragma unroll
+    for (int i = 0; i < LN; ++i) {
+      auto at = [&](L a) -> float {
+        if constexpr (N == 1) return a.v;
+        else return i ? a.v.y : a.v.x;
+      };
+      const int j = j0 + i;
+      const float rh = at(r.hi), rl = at(r.lo), inv = rcp_estimate(rh);
+      float m = 0.f;
+#pragma unroll
+      for (int k = 0; k < 9; ++k) m = fmaxf(m, fabsf(at(g[k])));
+      bool holds = m <= 0.09375f;
+      // quotient: an estimate and its remainder, rounded once
+      auto div = [&](const Sum3<L> &a) {
+        const float ah = at(a.hi), q = __fmul_rn(ah, inv);
+        const float rem = __fadd_rn(__fmaf_rn(-q, rh, ah), __fmaf_rn(-q, rl, at(a.lo)));
+        const float w = __fmaf_rn(rem, inv, q);
+        holds = holds && (fabsf(w) > 0x1p-100f || (ah == 0.f && at(a.lo) == 0.f));  // false for NaN
+        return w;
+      };
+      o[0].s[j] = rh;
+      o[1].s[j] = div(jx);
+      o[2].s[j] = div(jy);
+      if (!holds) {
+        const float3 t = double_moments(f[0][j], f[1][j], f[2][j], f[3][j], f[4][j], f[5][j], f[6][j], f[7][j], f[8][j], p.U);
+        o[0].s[j] = t.x;
+        o[1].s[j] = t.y;
+        o[2].s[j] = t.z;
+      }
+      if (link_mask(p, x + j, y) & LM_SOLID) {
+        o[0].s[j] = 1.f;
+        o[1].s[j] = o[2].s[j] = 0.f;
+      }
+    }
   }
   const size_t at = (size_t)row * p.nx + x;
   *reinterpret_cast<Out *>(rho + at) = o[0];
