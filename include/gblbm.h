@@ -76,9 +76,11 @@ extern "C" {
 #define LBM_KERNEL_AUTO 0   /* the library's choice: the storage type's default kernel (which
                                lbm_get_kernel names); with float storage, no explicit shape and
                                no CTAs per SM given, two steps at a time run in one pass over
-                               memory, up to 64 per launch (bit-identical; single lattices
-                               with either bounce-back, and batches), and an odd step on the
-                               default kernel */
+                               memory, up to 64 per launch (single lattices with either
+                               bounce-back, and batches), and an odd step on the default
+                               kernel.  The populations are bit-identical; a force is a sum
+                               in double of the same links in another order, the same bits
+                               wherever that sum is exact */
 #define LBM_KERNEL_DIRECT 1 /* one thread per cell, loads straight from HBM */
 #define LBM_KERNEL_TMA 2    /* persistent; bulk-async (TMA) row staging */
 #define LBM_KERNEL_TMA_BULK 3 /* TMA row staging and TMA bulk stores of the new rows

@@ -454,24 +454,6 @@ __device__ __forceinline__ void boundaries(C h[9], int xe, int y, const StepPara
   if (xe == 0) inlet<C>(h, U);
 }
 
-// A sum of floats kept to twice their precision (two-sum, Knuth), for the few
-// places that need more than float: this chip does about two double operations
-// per clock and SM, sixty times fewer than float ones.
-struct Sum2 {
-  float hi = 0.f, lo = 0.f;
-  __device__ __forceinline__ void add(float v) {
-    const float t = __fadd_rn(hi, v), z = __fsub_rn(t, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(v, z)));
-    hi = t;
-  }
-  // hi becomes the float nearest to the sum
-  __device__ __forceinline__ void normalize() {
-    const float t = __fadd_rn(hi, lo);
-    lo = __fsub_rn(lo, __fsub_rn(t, hi));
-    hi = t;
-  }
-};
-
 // ---- lane arithmetic -------------------------------------------------------
 // The collisions are written once over a lane type: LF (one node, float),
 // LD (one node, double) or LF2 (two nodes in packed FP32 instructions,

@@ -88,6 +88,41 @@ __device__ __forceinline__ void set_elem(float2 &v, int j, float s) {
   else v.x = s;
 }
 
+// Force sums of a row's links.  A double operation costs an SM 16 clocks a warp and a
+// long wait, so a row is added in pairs of floats, and its sums go to the double totals
+// once.  The pairs lose nothing while the terms lie within a factor of 2^15: up to 32 of
+// them are multiples of the smallest one's last bit, their rounding errors below 2^-14 of
+// the largest, and the sum of those fits a float's 24 bits.  Rows with other terms, with
+// infinities or near the ends of the float range are added in double.
+struct LinkSum {
+  LF xh{}, xl{}, yh{}, yl{};
+  uint32_t most = 0, least = 0xffffffffu;  // largest term's bits; smallest nonzero one's, less 1
+  __device__ __forceinline__ void see(float t) {
+    const uint32_t bits = __float_as_uint(fabsf(t));
+    most = max(most, bits);
+    least = min(least, bits - 1u);
+  }
+  __device__ __forceinline__ void add(int k, float t) {  // along c_k
+    LF e;
+    if (CX(k)) {
+      xh = two_sum(xh, LF{CX(k) > 0 ? t : -t}, e);
+      xl = xl + e;
+    }
+    if (CY(k)) {
+      yh = two_sum(yh, LF{CY(k) > 0 ? t : -t}, e);
+      yl = yl + e;
+    }
+    see(t);
+  }
+  __device__ __forceinline__ bool exact() const {
+    return (most >> 23) < 248u && (most >> 23) <= ((least + 1u) >> 23) + 15u;
+  }
+  __device__ __forceinline__ void to(double &fx, double &fy) const {
+    fx += (double)xh.v + (double)xl.v;
+    fy += (double)yh.v + (double)yl.v;
+  }
+};
+
 // The wall rules of boundaries() for a node of the bottom or top row.
 __device__ __forceinline__ void pair_wall(int bc, bool bottom, float U, float (&v)[9]) {
   if (bc == BC_FREESLIP) {
@@ -243,8 +278,7 @@ __global__ void __launch_bounds__(NW * 32, 1)
     const Coef<LP2> cf = make_coef<LP2>(p);
     const float U = (float)p.U;
     uint32_t worst = 0;                             // largest |u|^2 seen, as bits
-    // this lane's links, per stage: a row's links are added in float pairs, the
-    // row's sum goes to the double total
+    // this lane's links, per stage
     double fx[2] = {0.0, 0.0}, fy[2] = {0.0, 0.0};
     int st = 0;                                     // stage of the current row's tile
     const bool map_cols = p.lx0 < base + kPairCols && p.lx0 + p.lw > base;  // the window meets the link map
@@ -276,7 +310,7 @@ __global__ void __launch_bounds__(NW * 32, 1)
     auto update = [&](float2 (&g)[9], int y, const uint32_t (&m)[2], bool links, const float2 (&own)[9], bool counts,
                       int s) {
       if (links) {
-        [[maybe_unused]] Sum2 sx, sy;  // interpolated links: the populations that leave and return
+        [[maybe_unused]] LinkSum sum;  // interpolated links: the populations that leave and return
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
           if (!__any_sync(0xffffffffu, (m[j] & LM_LINKS) != 0)) continue;
@@ -305,18 +339,27 @@ __global__ void __launch_bounds__(NW * 32, 1)
                 }
                 if (CX(k)) r += (float)(-6.0 * WD(k) * CX(k)) * U * wref;
                 set_elem(g[k], j, r);
-                sx.add(CX(OPP(k)) * hi);
-                sx.add(CX(OPP(k)) * r);
-                sy.add(CY(OPP(k)) * hi);
-                sy.add(CY(OPP(k)) * r);
+                sum.add(OPP(k), hi);
+                sum.add(OPP(k), r);
               }
             }
           }
         }
         if constexpr (INTERP) {
           if (counts && mine) {
-            fx[s] += (double)sx.hi + (double)sx.lo;
-            fy[s] += (double)sy.hi + (double)sy.lo;
+            if (sum.exact()) {
+              sum.to(fx[s], fy[s]);
+            } else {
+#pragma unroll 1
+              for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int k = 1; k < 9; ++k)
+                  if ((j ? m[1] : m[0]) & (1u << k)) {
+                    const double t = (double)elem(own[OPP(k)], j) + (double)elem(g[k], j);
+                    if (CX(k)) fx[s] += CX(k) < 0 ? t : -t;
+                    if (CY(k)) fy[s] += CY(k) < 0 ? t : -t;
+                  }
+            }
           }
         }
       }
@@ -368,18 +411,48 @@ __global__ void __launch_bounds__(NW * 32, 1)
         }
         if constexpr (!INTERP) {
           if (counts) {  // half-way links: the population leaves and returns (the factor 2 comes last)
-            Sum2 sx, sy;
+            // Per node one value for each pair of opposite directions (both seldom hold a
+            // link), and no branch for a direction without links.
+            float d[2][4];
+            uint32_t both = 0;
 #pragma unroll
-            for (int k = 1; k < 9; ++k)
+            for (int j = 0; j < 2; ++j) {
+              const uint32_t mj = mine ? m[j] : 0u;
+              auto of = [&](int k) { return mj & (1u << OPP(k)) ? elem(g[k], j) : 0.f; };
+              both |= mj & (mj >> 2) & 0x66u;  // directions 1 and 3, 2 and 4, 5 and 7, 6 and 8
+              d[j][0] = of(1) - of(3);
+              d[j][1] = of(2) - of(4);
+              d[j][2] = of(5) - of(7);
+              d[j][3] = of(6) - of(8);
+            }
+            LF t[4], l[4], e;  // the two nodes' values added
+            LinkSum sum;
 #pragma unroll
-              for (int j = 0; j < 2; ++j) {
-                const float t = m[j] & (1u << OPP(k)) ? elem(g[k], j) : 0.f;
-                if (CX(k)) sx.add(CX(k) > 0 ? t : -t);
-                if (CY(k)) sy.add(CY(k) > 0 ? t : -t);
-              }
-            if (mine) {
-              fx[s] += (double)sx.hi + (double)sx.lo;
-              fy[s] += (double)sy.hi + (double)sy.lo;
+            for (int c = 0; c < 4; ++c) {
+              t[c] = two_sum(LF{d[0][c]}, LF{d[1][c]}, l[c]);
+              sum.see(d[0][c]);
+              sum.see(d[1][c]);
+            }
+            sum.xh = two_sum(t[0], t[2], e);
+            sum.xl = (l[0] + l[2]) + e;
+            sum.xh = two_diff(sum.xh, t[3], e);
+            sum.xl = sum.xl + (e - l[3]);
+            sum.yh = two_sum(t[1], t[2], e);
+            sum.yl = (l[1] + l[2]) + e;
+            sum.yh = two_sum(sum.yh, t[3], e);
+            sum.yl = sum.yl + (e + l[3]);
+            if (!both && sum.exact()) {
+              sum.to(fx[s], fy[s]);
+            } else {
+#pragma unroll 1
+              for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int k = 1; k < 9; ++k)
+                  if ((mine ? (j ? m[1] : m[0]) : 0u) & (1u << OPP(k))) {
+                    const double t = j ? g[k].y : g[k].x;
+                    if (CX(k)) fx[s] += CX(k) > 0 ? t : -t;
+                    if (CY(k)) fy[s] += CY(k) > 0 ? t : -t;
+                  }
             }
           }
         }
