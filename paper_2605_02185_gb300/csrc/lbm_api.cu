@@ -25,6 +25,18 @@ namespace {
 
 constexpr int kLayoutParts = 11;
 
+// The most row tiles of one row that the columns [x0, x1] meet, over the tile widths a
+// context of this storage may be given (a body that lies in one tile of one width may
+// cross a boundary of another's).
+int most_tiles(int storage, int x0, int x1) {
+  int most = 1;
+  auto see = [&](int seg) { most = std::max(most, x1 / seg - x0 / seg + 1); };
+  see(kDirectThreads);
+  for (const TmaShape &t : kTmaShapes) see(ops_for(storage)->tma_pair * t.ncw * 32 * t.cpt);
+  for (const TmaShape &t : kTmaBulkShapes) see(t.ncw * 32 * t.cpt);
+  return most;
+}
+
 size_t layout(const lbm_opts *o, const Geometry &g, int *pitch_out, size_t offs[kLayoutParts], int *slot_cap_out,
               int *band_rows_out) {
   const int elem = elem_size(o->storage);
@@ -33,7 +45,7 @@ size_t layout(const lbm_opts *o, const Geometry &g, int *pitch_out, size_t offs[
   const size_t lmap = align_up(std::max<size_t>(g.lmap.size(), 1) * sizeof(uint16_t), kAlign) +
                       align_up(g.qmap.size() * sizeof(float), kAlign);  // link fractions follow the map
   int slot_cap = 1;
-  if (g.fx1 >= g.fx0) slot_cap = (g.fy1 - g.fy0 + 1) * (g.fx1 / 256 - g.fx0 / 256 + 1);
+  if (g.fx1 >= g.fx0) slot_cap = (g.fy1 - g.fy0 + 1) * most_tiles(o->storage, g.fx0, g.fx1);
   const size_t slots = align_up((size_t)slot_cap * sizeof(double2), kAlign);
   const long long cap = o->history_capacity > 0 ? o->history_capacity : (1ll << 20);
   const size_t hist = align_up((size_t)cap * 2 * sizeof(double), kAlign);

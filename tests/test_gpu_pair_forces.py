@@ -78,3 +78,22 @@ def test_infinite_links():
     got = run(nx, ny, mask, pops, 2)
     assert not np.all(np.isfinite(ref[1]))
     assert np.array_equal(ref[1], got[1], equal_nan=True)
+
+
+@pytest.mark.parametrize("bounce", [lbm.LBM_BOUNCE_HALFWAY, lbm.LBM_BOUNCE_INTERPOLATED], ids=["half", "interp"])
+def test_wide_body(bounce):
+    # about a thousand links below 0.1: a double sum in another order differs by less than
+    # 1000 x 2^-53 of the sum of magnitudes, 2 x 1000 x 0.1
+    wl = W.random_case(1601, 300, seed=7, bc=W.BC_FREESLIP, D=140, U=0.04)
+    out = []
+    for kernel in (lbm.LBM_KERNEL_DIRECT, lbm.LBM_KERNEL_AUTO):
+        lat = lbm.lattice_for(wl, kernel=kernel, bounce=bounce)
+        try:
+            lat.init_fields(*wl.initial_fields())
+            lat.step(70)
+            lat.sync()
+            out.append((lat.get_populations(), lat.forces_raw()))
+        finally:
+            lat.close()
+    assert np.array_equal(out[0][0].view(np.uint32), out[1][0].view(np.uint32))
+    assert np.abs(out[0][1] - out[1][1]).max() <= 1000 * 2.0 ** -53 * 200
