@@ -1138,7 +1138,11 @@ __global__ void init_device_kernel(S *__restrict__ A, StepParams p, const float 
       continue;
     }
     const double r = rho[i], ux = u[i], uy = v[i];
-    const double uu15 = 1.5 * (ux * ux + uy * uy);
+    // infinite velocities: the formula's answer, to which every direction's zero
+    // components of c add zero times infinity
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+    const bool finite = fabsf(u[i]) < __int_as_float(0x7f800000) && fabsf(v[i]) < __int_as_float(0x7f800000);
+    const double uu15 = finite ? 1.5 * (ux * ux + uy * uy) : nan;
     double dudx = 0.0, dudy = 0.0, dvdx = 0.0, dvdy = 0.0;
     if (with_noneq) {
       dudx = diff1(u, p, x, y, 1, 0);
@@ -1168,6 +1172,7 @@ __global__ void init_device_kernel(S *__restrict__ A, StepParams p, const float 
       qp = nd * (dd + shear);
       qm = nd * (dd - shear);
       qr = n3 * WD(0) * r * (q0 * dudx + q0 * dvdy);
+      if ((__double2hiint(shear) & 0x7ff00000) == 0x7ff00000) qx = qy = qr = nan;  // c_x c_y = 0 times it
     }
     const double wa = WD(1) * r, wd = WD(5) * r, cp = ux + uy, cm = uy - ux;
     put(0, WD(0) * r, 0.0, 0.0, qr);
