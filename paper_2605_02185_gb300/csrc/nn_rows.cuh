@@ -366,22 +366,9 @@ cudaError_t launch_rows(const void *x, int xs, const void *w, const float *bias,
   using Lay = RowLayout<BN, CIN, SLOTS>;
   static_assert(Lay::ALLOC <= 227 * 1024, "shared memory");
   auto kern = conv_rows_kernel<BN, CIN, SLOTS>;
-  static int per_sm = 0;
-  if (!per_sm) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay::ALLOC);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    if (e != cudaSuccess) return e;
-    cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, kern);
-    if (e != cudaSuccess) return e;
-    const int regs = (fa.numRegs + 7) / 8 * 8;
-    int n = 233472 / (Lay::ALLOC + 1024);
-    n = n < 65536 / (regs * kRowThreads) ? n : 65536 / (regs * kRowThreads);
-    n = n < tmem_ctas(Lay::NCOLS) ? n : tmem_ctas(Lay::NCOLS);
-    if (n < 1) return cudaErrorInvalidConfiguration;
-    per_sm = n;
-  }
+  static PerDevice resident;
+  const int per_sm = resident.get(current_device(), [&] { return resident_ctas(kern, Lay::ALLOC, kRowThreads, Lay::NCOLS); });
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const long long units = (long long)N * ((W + kTileM - 1) / kTileM) * H;
   const long long most = (long long)per_sm * sm_count();
   kern<<<(int)(units < most ? units : most), kRowThreads, Lay::ALLOC, st>>>(

@@ -31,6 +31,7 @@
 #include <cudaTypedefs.h>
 #include <stdint.h>
 
+#include "nn_per_device.h"
 #include "nn_tc.h"
 
 namespace gbnn_tc {
@@ -663,14 +664,35 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
+int current_device() {
+  int dev = -1;
+  return cudaGetDevice(&dev) == cudaSuccess ? dev : -1;
+}
+
 int sm_count() {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      sms = 148;
-  }
-  return sms;
+  static PerDevice count;
+  const int dev = current_device();
+  return count.get(dev, [&] {
+    int sms = 0;
+    return cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? sms : 148;
+  });
+}
+
+// Let `kern` have its shared memory on the current device; the CTAs of it an SM holds
+// (0 on an error): shared memory (228 KB per SM, 1 KB reserved per CTA), registers (64K
+// per SM, allocated in units of 8 per thread), threads, and the tensor-memory columns.
+template <class Kernel>
+int resident_ctas(Kernel kern, int smem, int threads, uint32_t columns) {
+  cudaFuncAttributes fa;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+      cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100) != cudaSuccess ||
+      cudaFuncGetAttributes(&fa, kern) != cudaSuccess)
+    return 0;
+  const int regs = (fa.numRegs + 7) / 8 * 8;
+  int n = 233472 / (smem + 1024);
+  n = n < 65536 / (regs * threads) ? n : 65536 / (regs * threads);
+  n = n < 2048 / threads ? n : 2048 / threads;
+  return n < tmem_ctas(columns) ? n : tmem_ctas(columns);
 }
 
 template <int BN, int CK, int STAGES>
@@ -678,26 +700,9 @@ cudaError_t launch(const CUtensorMap &tx, const CUtensorMap &tw, const float *bi
                    int ms, int N, int H, int W, int cin, int nchunks, int relu, cudaStream_t st) {
   using Lay = TcLayout<BN, CK, STAGES>;
   auto kern = conv_tc_kernel<BN, CK, STAGES>;
-  static int per_sm = 0;
-  if (!per_sm) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay::ALLOC);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    if (e != cudaSuccess) return e;
-    cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, kern);
-    if (e != cudaSuccess) return e;
-    // resident CTAs per SM: shared memory (228 KB per SM, 1 KB reserved per
-    // CTA), registers (64K per SM, allocated in units of 8 per thread),
-    // threads, and the tensor-memory columns
-    const int regs = (fa.numRegs + 7) / 8 * 8;
-    int n = 233472 / (Lay::ALLOC + 1024);
-    n = n < 65536 / (regs * kThreads) ? n : 65536 / (regs * kThreads);
-    n = n < 2048 / kThreads ? n : 2048 / kThreads;
-    n = n < tmem_ctas(Lay::NCOLS) ? n : tmem_ctas(Lay::NCOLS);
-    if (n < 1) return cudaErrorInvalidConfiguration;
-    per_sm = n;
-  }
+  static PerDevice resident;
+  const int per_sm = resident.get(current_device(), [&] { return resident_ctas(kern, Lay::ALLOC, kThreads, Lay::NCOLS); });
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const long long ntiles = (long long)N * H * ((W + kTileM - 1) / kTileM) * nchunks;
   if (ntiles > 0x7fffffff) return cudaErrorInvalidValue;
   const int grid = (int)(ntiles < (long long)per_sm * sm_count() ? ntiles : (long long)per_sm * sm_count());
@@ -777,12 +782,11 @@ cudaError_t launch_wgrad(const CUtensorMap &tx, const CUtensorMap &tg, float *gw
                          int nblocks, int mtiles, long long ksteps, int splits, cudaStream_t st) {
   using Lay = WgLayout<BN, STAGES>;
   auto kern = wgrad_tc_kernel<BN, STAGES>;
-  static bool prepared = false;
-  if (!prepared) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay::ALLOC);
-    if (e != cudaSuccess) return e;
-    prepared = true;
-  }
+  static PerDevice prepared;
+  if (prepared.get(current_device(), [&] {
+        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay::ALLOC) == cudaSuccess ? 1 : 0;
+      }) < 1)
+    return cudaErrorInvalidConfiguration;
   const long long per = (ksteps + splits - 1) / splits;
   const int nsplit = (int)((ksteps + per - 1) / per);
   kern<<<dim3(mtiles, nsplit), kThreads, Lay::ALLOC, st>>>(tx, tg, gw, H, W, cin, cout, nblocks, ksteps, per);
