@@ -377,14 +377,15 @@ cudaError_t launch_rows(const void *x, int xs, const void *w, const float *bias,
 }
 
 // kNotEligible where there is no row kernel for the channel counts or the
-// alignment; arguments as conv_fwd.  Layers of 8 channels only where `eight`: a
+// alignment, or where the image is too small for it (nn_rows_rule.h); arguments as conv_fwd.  Layers of 8 channels only where `eight`: a
 // caller that requires the tensor-core kernels by name is refused them.
 int conv_rows(const void *x, int xs, const void *w, const float *bias, void *y, int ys, const void *mask, int ms, int N,
               int H, int W, int cin, int cout, int relu, bool eight, cudaStream_t st) {
   if (!eight && (cin == 8 || cout == 8)) return kNotEligible;
   if (xs % 8 || ys % 8 || (uintptr_t)x % 16 || (uintptr_t)w % 16 || (uintptr_t)y % 16) return kNotEligible;
   if (mask && ((uintptr_t)mask % 16 || ms % 8)) return kNotEligible;
-  if ((long long)N * ((W + kTileM - 1) / kTileM) > 0x7fffffff) return kNotEligible;
+  const long long columns = (long long)N * ((W + kTileM - 1) / kTileM);
+  if (columns > 0x7fffffff || !rows_pay(cin, cout, columns * H, sm_count())) return kNotEligible;
   cudaError_t e;
 #define GBNN_ROWS_CASE(CIN_, COUT_, BN_, SLOTS_)                                                            \
   if (cin == CIN_ && cout == COUT_)                                                                         \

@@ -32,6 +32,7 @@
 #include <stdint.h>
 
 #include "nn_per_device.h"
+#include "nn_rows_rule.h"
 #include "nn_tc.h"
 
 namespace gbnn_tc {
