@@ -51,7 +51,7 @@ size_t pair_region_bytes(int cells, int slots, int cases) {
 int pair_plan(const std::vector<PairLattice> &lattices, int sms, void *region, int cells_cap, int slots_cap,
               cudaStream_t st, PairParams *q, int *grid) {
   *grid = 0;
-  const int warps = sms * kPairWarps;
+  int warps = sms * kPairWarps;
   std::vector<Window> win;
   for (size_t l = 0; l < lattices.size(); ++l) {
     const PairLattice &t = lattices[l];
@@ -66,6 +66,12 @@ int pair_plan(const std::vector<PairLattice> &lattices, int sms, void *region, i
       win.push_back(v);
     }
   }
+  // A lattice of about as many rows as half the warps leaves the other half: it gains 1 %
+  // from the rest (400 x 200, 1,400 rows: 4.78 us a step, with 1,216 warps 4.83), and the
+  // launches of two such lattices on two streams then run at the same time (9.16 and 5.49
+  // us a step of both; four of them 18.5 and 10.6).  With 3,300 rows, 600 x 300, half the
+  // warps would cost it 10 %.
+  if (lattices.size() == 1 && (long long)win.size() * lattices[0].ny * 5 <= 3ll * warps) warps /= 2;
   // One cell per warp where that can be: every window is cut into bands of rows
   // of equal cost, as cheap as the number of warps allows.
   auto bands = [&](const Window &v, double cost) {

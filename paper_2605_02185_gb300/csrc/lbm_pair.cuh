@@ -32,6 +32,8 @@
 // 3200 x 1600 66.4 -> 38.3, 8000 x 4000 357 -> 235, 16000 x 8000 1416 -> 1102.
 #pragma once
 
+#include <algorithm>
+
 #include "lbm_kernels.cuh"
 
 namespace gblbm {
@@ -572,8 +574,11 @@ cudaError_t pair_one(int grid, float *buf0, float *buf1, const StepParams &p, co
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(NW * 32);
-  cfg.dynamicSmemBytes = smem;
+  // only the warps that get a cell, with their rings: launches of several small lattices
+  // on streams of their own then share the SMs
+  const int per = std::min(NW, (q.ncells + grid - 1) / grid);
+  cfg.blockDim = dim3(per * 32);
+  cfg.dynamicSmemBytes = per * PairLayout<NW, STAGES>::WARP;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
