@@ -335,7 +335,11 @@ def lbm_probe_stochastic_round(storage: int, x_ptr: int, salt_ptr: int, out_ptr:
            "lbm_probe_stochastic_round")
 
 
-def lbm_set_kernel(h, kernel: int, consumer_warps=0, cells_per_thread=0, stages=0, ctas_per_sm=1):
+def lbm_set_kernel(h, kernel: int, consumer_warps=0, cells_per_thread=0, stages=0, ctas_per_sm=None):
+    """``ctas_per_sm``: 0 leaves it to the library; by default 1 for a named kernel and 0 for
+    LBM_KERNEL_AUTO, for which any other number counts as a choice of the one-step kernel."""
+    if ctas_per_sm is None:
+        ctas_per_sm = 0 if int(kernel) == LBM_KERNEL_AUTO else 1
     _check(load_library().lbm_set_kernel(h, int(kernel), int(consumer_warps), int(cells_per_thread), int(stages),
                                          int(ctas_per_sm)), "lbm_set_kernel")
 
