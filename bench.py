@@ -67,10 +67,17 @@ def kernel_digest() -> str:
     import hashlib
     h = hashlib.sha256()
     d = os.path.join(ROOT, "paper_2605_02185_gb300", "csrc")
-    for name in ("lbm_device.cuh", "lbm_kernels.cuh"):
+    for name in ("lbm_device.cuh", "lbm_kernels.cuh", "lbm_pair.cuh", "lbm_pair.cu"):
         with open(os.path.join(d, name), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
+
+
+def bytes_per_step(bytes_pass: float, steps: int, steps_per_pass: int) -> float:
+    """Mean algorithmic bytes of each of ``steps`` steps: those left over from the
+    passes are a pass each."""
+    passes = steps // steps_per_pass + steps % steps_per_pass
+    return bytes_pass * passes / max(steps, 1)
 
 
 def measured_peaks():
@@ -303,15 +310,13 @@ def run_ours(args, workload):
     t_max = max_over_ranks(t_ms / 1e3, device)
     value = whole_job_glups(nx * ny, args.steps, world, t_max)
     per_launch_s = (t_ms / 1e3) / args.steps
-    # the library's own choice for float storage takes two steps per pass over
-    # memory: a step's share is half of one read and one write of the populations
-    two_step = args.kernel == "auto" and args.storage == "f32" and shape is None and not args.ctas_per_sm
-    bytes_step = lat.bytes_per_step() * (0.5 if two_step else 1.0)
+    per_pass = lat.steps_per_pass()
+    bytes_step = bytes_per_step(lat.bytes_per_step(), args.steps, per_pass)
     peak, peak_src = measured_peaks()
     achieved = bytes_step / per_launch_s / 1e9
     digest = kernel_digest()
     traffic = None
-    if NCU_TRAFFIC["digest"] == digest and args.storage in NCU_TRAFFIC["bytes_per_node"]:
+    if per_pass == 1 and NCU_TRAFFIC["digest"] == digest and args.storage in NCU_TRAFFIC["bytes_per_node"]:
         traffic = NCU_TRAFFIC["bytes_per_node"][args.storage] * nx * ny
     info = lat.kernel_info()
 
@@ -356,12 +361,12 @@ def run_ours(args, workload):
                    "collision": args.collision,
                    "kernel": info, "parallelism": f"replicas x{world}" if world > 1 else "single GPU",
                    "gpu": torch.cuda.get_device_name(device), "seed": workload.seed,
-                   "steps_per_pass": 2 if two_step else 1,
+                   "steps_per_pass": per_pass,
                    "l2": f"{9 * lbm.ELEM_BYTES[storage] * nx * ny / 1e9:.1f} GB of populations read per pass, far "
                          "above the 129 MB L2: no flush needed"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic, "peak_source": peak_src,
-                     "algorithmic_bytes_per_launch": bytes_step},
+                     "algorithmic_bytes_per_step": bytes_step},
         "e2e": e2e,
         "gpu_launches": int(launches),
         "clocks": clocks,
@@ -427,8 +432,8 @@ def extras(args, workload, device, stream):
     out["batch"] = {"workload": "64 cylinder cases, Re log-uniform in [60, 200], D in {20, 30, 40, 60}, "
                                 "40D x 20D, U = 0.05, free-slip, MRT (Eq. 6)",
                     "nodes": nodes, "steps": steps, "glups": nodes * steps / dt / 1e9,
-                    # two steps per pass: half of a read and a write per step
-                    "roofline_frac": 0.5 * bytes_step * steps / dt / 1e9 / peak, "steps_per_pass": 2,
+                    "roofline_frac": bytes_per_step(bytes_step, steps, b.steps_per_pass()) * steps / dt / 1e9 / peak,
+                    "steps_per_pass": b.steps_per_pass(),
                     "kernel": b.kernel_info()}
     b.close()
     del b
@@ -509,7 +514,7 @@ def run_batch(args):
     # the same work either way, so the timing stands and the cases are named.
     unstable = [w.name for c, w in enumerate(cases) if b.case_status(c) == lbm.LBM_ERR_UNSTABLE]
     t_batch = e0.elapsed_time(e1) / 1e3
-    info = b.kernel_info()
+    info, per_pass = b.kernel_info(), b.steps_per_pass()
     b.close()
     del b
     torch.cuda.empty_cache()
@@ -532,8 +537,7 @@ def run_batch(args):
     value = whole_job_glups(nodes, args.steps, world, t_max)
     seq = nodes * args.steps / t_seq / 1e9
     peak, src = measured_peaks()
-    two_step = tuned is None or tuned["kind"] == autotune.AUTO  # half of a read and a write per step
-    bytes_step *= 0.5 if two_step else 1.0
+    bytes_step = bytes_per_step(bytes_step, args.steps, per_pass)
     achieved = bytes_step / (t_batch / args.steps) / 1e9
     if rank == 0:
         print(json.dumps({
@@ -543,13 +547,13 @@ def run_batch(args):
             "vs_baseline": None, "dtype": "f32", "data": "synthetic",
             "config": {"workload": f"batch of {len(cases)} cylinder cases, Re in [60,200], D in {{20,30,40,60}}, "
                                    f"40D x 20D, U = 0.05, free-slip", "nodes": nodes, "kernel": info,
-                       "steps_per_pass": 2 if two_step else 1, "collision": args.collision,
+                       "steps_per_pass": per_pass, "collision": args.collision,
                        "tuned": tuned},
             "sequential": {"value": seq, "unit": UNIT, "note": "same cases one after another, each a "
                                                                 "single lattice"},
             "speedup_vs_sequential": value / seq / world,
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                         "traffic": None, "peak_source": src, "algorithmic_bytes_per_launch": bytes_step},
+                         "traffic": None, "peak_source": src, "algorithmic_bytes_per_step": bytes_step},
             "unstable_cases": unstable, "gpu_launches": int(launches), "clocks": clocks}), flush=True)
     return 0
 

@@ -80,7 +80,13 @@ extern "C" {
                                bounce-back, and batches), and an odd step on the default
                                kernel.  The populations are bit-identical; a force is a sum
                                in double of the same links in another order, the same bits
-                               wherever that sum is exact */
+                               wherever that sum is exact.  lbm_steps_per_pass tells whether
+                               a lattice is taken; left to the default kernel are some
+                               whose body spans a third of the width or more, and those
+                               wider than about 490,000 nodes.  Lattices of 150,000 to
+                               300,000 nodes stepped on three or more streams at a time are
+                               faster on LBM_KERNEL_TMA (or in a batch): the launches of
+                               two steps per pass follow one another */
 #define LBM_KERNEL_DIRECT 1 /* one thread per cell, loads straight from HBM */
 #define LBM_KERNEL_TMA 2    /* persistent; bulk-async (TMA) row staging */
 #define LBM_KERNEL_TMA_BULK 3 /* TMA row staging and TMA bulk stores of the new rows
@@ -256,9 +262,13 @@ int lbm_get_window(lbm_ctx *ctx, int x0, int y0, int w, int h, void *dst);
 /* Switch the step kernel (LBM_KERNEL_*) and its shape; re-captures graphs. */
 int lbm_set_kernel(lbm_ctx *ctx, int kernel, int consumer_warps, int cells_per_thread, int stages,
                    int ctas_per_sm);
-/* The kernel shape in use: kernel, consumer warps, cells/thread, stages,
- * CTAs per SM, grid size (CTAs) -- 6 ints. */
+/* The shape of the one-step kernel in use: kernel, consumer warps, cells/thread,
+ * stages, CTAs per SM, grid size (CTAs) -- 6 ints.  Where lbm_steps_per_pass
+ * gives 2 it takes the steps that are left over from the pairs. */
 int lbm_get_kernel(lbm_ctx *ctx, int *out6);
+/* Steps that one pass over memory takes: 2 where LBM_KERNEL_AUTO runs two at a
+ * time, else 1. */
+int lbm_steps_per_pass(lbm_ctx *ctx, int *steps);
 
 /* Host only (no GPU call): the kernel, consumer warps, cells/thread, stages
  * and CTAs per SM (5 ints into out5) that lbm_create_ex picks for *opts
@@ -301,8 +311,9 @@ int lbm_get_stream(lbm_ctx *ctx, void **stream);
  * launch of several steps counts 2, with its force reduction). */
 int lbm_launch_count(lbm_ctx *ctx, int64_t *count);
 
-/* Algorithmic bytes one step moves through HBM: 2 * 9 * element size per
- * node (read f*(n-1), write f*(n)). */
+/* Algorithmic bytes one pass over memory moves through HBM: 2 * 9 * element
+ * size per node (read f*(n-1), write f*(n); where lbm_steps_per_pass gives 2,
+ * f*(n+1), so that a step's share is half). */
 int lbm_bytes_per_step(lbm_ctx *ctx, double *bytes);
 
 /* One step WITHOUT ANY ALLOCATION, for callers that may not allocate device
@@ -370,12 +381,14 @@ int lbm_batch_sync(lbm_batch *batch);
 int lbm_batch_set_kernel(lbm_batch *batch, int kernel, int consumer_warps, int cells_per_thread, int stages,
                          int ctas_per_sm);
 int lbm_batch_get_kernel(lbm_batch *batch, int *out6);
+int lbm_batch_steps_per_pass(lbm_batch *batch, int *steps); /* as lbm_steps_per_pass */
 /* lbm_set_fault_injection for a batch on LBM_KERNEL_TMA (LBM_ERR_ARG
  * otherwise): row tile `tile` of case c; the wait limit holds for every case. */
 int lbm_batch_set_fault_injection(lbm_batch *batch, int c, int64_t tile, double wait_seconds);
 int lbm_batch_get_stream(lbm_batch *batch, void **stream);
 int lbm_batch_launch_count(lbm_batch *batch, int64_t *count);
-/* Total nodes of all cases, and the algorithmic HBM bytes of one batch step. */
+/* Total nodes of all cases, and the algorithmic HBM bytes of one pass over them
+ * (as lbm_bytes_per_step). */
 int lbm_batch_nodes(lbm_batch *batch, int64_t *nodes, double *bytes_per_step);
 
 /* Diagnostic (no counterpart in the paper): -1/x as the float collisions

@@ -715,6 +715,12 @@ int lbm_get_kernel(lbm_ctx *c, int *out6) {
   return LBM_OK;
 }
 
+int lbm_steps_per_pass(lbm_ctx *c, int *steps) {
+  if (!c || !steps) return LBM_ERR_ARG;
+  *steps = c->pair ? 2 : 1;
+  return LBM_OK;
+}
+
 int lbm_kernel_shapes(int *out, int cap, int *count) {
   if (!count || cap < 0 || (cap > 0 && !out)) return LBM_ERR_ARG;
   *count = kNumTmaShapes;

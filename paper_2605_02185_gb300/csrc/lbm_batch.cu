@@ -398,6 +398,12 @@ int lbm_batch_get_kernel(lbm_batch *b, int *out6) {
   return LBM_OK;
 }
 
+int lbm_batch_steps_per_pass(lbm_batch *b, int *steps) {
+  if (!b || !steps) return LBM_ERR_ARG;
+  *steps = b->pair ? 2 : 1;
+  return LBM_OK;
+}
+
 int lbm_batch_get_stream(lbm_batch *b, void **stream) {
   if (!b || !stream) return LBM_ERR_ARG;
   *stream = (void *)b->stream;

@@ -102,6 +102,7 @@ def load_library(path: str | None = None):
         "lbm_get_window": (i, [vp, i, i, i, i, vp]),
         "lbm_set_kernel": (i, [vp, i, i, i, i, i]),
         "lbm_get_kernel": (i, [vp, vp]),
+        "lbm_steps_per_pass": (i, [vp, ctypes.POINTER(i)]),
         "lbm_default_kernel": (i, [ctypes.POINTER(lbm_opts), vp]),
         "lbm_kernel_shapes": (i, [vp, i, ctypes.POINTER(i)]),
         "lbm_kernel_shapes_for": (i, [i, vp, i, ctypes.POINTER(i)]),
@@ -125,6 +126,7 @@ def load_library(path: str | None = None):
         "lbm_batch_set_kernel": (i, [vp, i, i, i, i, i]),
         "lbm_batch_set_fault_injection": (i, [vp, i, i64, d]),
         "lbm_batch_get_kernel": (i, [vp, vp]),
+        "lbm_batch_steps_per_pass": (i, [vp, ctypes.POINTER(i)]),
         "lbm_batch_get_stream": (i, [vp, ctypes.POINTER(vp)]),
         "lbm_batch_launch_count": (i, [vp, ctypes.POINTER(i64)]),
         "lbm_batch_nodes": (i, [vp, ctypes.POINTER(i64), ctypes.POINTER(d)]),
@@ -351,6 +353,12 @@ def lbm_get_kernel(h) -> dict:
     return dict(zip(keys, (int(v) for v in out)))
 
 
+def lbm_steps_per_pass(h) -> int:
+    n = ctypes.c_int()
+    _check(load_library().lbm_steps_per_pass(h, ctypes.byref(n)), "lbm_steps_per_pass")
+    return int(n.value)
+
+
 def lbm_default_kernel(opts: lbm_opts) -> dict:
     out = np.zeros(5, np.int32)
     _check(load_library().lbm_default_kernel(ctypes.byref(opts), _p(out)), "lbm_default_kernel")
@@ -497,6 +505,9 @@ class Lattice:
     def kernel_info(self) -> dict:
         return lbm_get_kernel(self.h)
 
+    def steps_per_pass(self) -> int:
+        return lbm_steps_per_pass(self.h)
+
     def launch_count(self) -> int:
         return lbm_launch_count(self.h)
 
@@ -582,6 +593,12 @@ def lbm_batch_get_kernel(h) -> dict:
     _check(load_library().lbm_batch_get_kernel(h, _p(out)), "lbm_batch_get_kernel")
     keys = ("kernel", "consumer_warps", "cells_per_thread", "stages", "ctas_per_sm", "grid")
     return dict(zip(keys, (int(v) for v in out)))
+
+
+def lbm_batch_steps_per_pass(h) -> int:
+    n = ctypes.c_int()
+    _check(load_library().lbm_batch_steps_per_pass(h, ctypes.byref(n)), "lbm_batch_steps_per_pass")
+    return int(n.value)
 
 
 def lbm_batch_launch_count(h) -> int:
@@ -696,6 +713,9 @@ class Batch:
 
     def kernel_info(self) -> dict:
         return lbm_batch_get_kernel(self.h)
+
+    def steps_per_pass(self) -> int:
+        return lbm_batch_steps_per_pass(self.h)
 
     def launch_count(self) -> int:
         return lbm_batch_launch_count(self.h)
