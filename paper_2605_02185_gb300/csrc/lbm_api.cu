@@ -37,7 +37,7 @@ int most_tiles(int storage, int x0, int x1) {
   return most;
 }
 
-size_t layout(const lbm_opts *o, const Geometry &g, int *pitch_out, size_t offs[kLayoutParts], int *slot_cap_out,
+size_t layout(const lbm_opts *o, const Geometry &g, bool pair_tables, int *pitch_out, size_t offs[kLayoutParts], int *slot_cap_out,
               int *band_rows_out) {
   const int elem = elem_size(o->storage);
   const int pitch = (int)align_up((size_t)o->nx, 64);
@@ -65,7 +65,7 @@ size_t layout(const lbm_opts *o, const Geometry &g, int *pitch_out, size_t offs[
   offs[6] = off; off += staging;
   offs[7] = off; off += wave_slots;
   offs[8] = off; off += wave_rows;
-  offs[9] = off; off += o->storage == LBM_F32 ? pair_region_bytes(kPairCellsSingle, kPairSlotsSingle, 1) : 0;
+  offs[9] = off; off += pair_tables && o->storage == LBM_F32 ? pair_region_bytes(kPairCellsSingle, kPairSlotsSingle, 1) : 0;
   offs[10] = off;
   *pitch_out = pitch;
   *slot_cap_out = slot_cap;
@@ -182,7 +182,7 @@ int configure_kernel(lbm_ctx *c, int kernel, int shape, int ctas_per_sm) {
 int configure_pair(lbm_ctx *c, bool automatic) {
   c->pair = false;
   c->pair_grid = 0;
-  if (!automatic || c->o.storage != LBM_F32 || c->kernel != LBM_KERNEL_TMA) return LBM_OK;
+  if (!automatic || !c->pair_region || c->o.storage != LBM_F32 || c->kernel != LBM_KERNEL_TMA) return LBM_OK;
   CK(pair_f32(0, nullptr, nullptr, c->p, c->pq, nullptr, 1, nullptr));
   int occ = 0;
   CK(pair_f32(0, nullptr, nullptr, c->p, c->pq, nullptr, 2, &occ));
@@ -285,23 +285,9 @@ int capture_graph(lbm_ctx *c) {
 
 }  // namespace
 
-extern "C" {
+namespace gblbm {
 
-int lbm_opts_default(lbm_opts *o) {
-  if (!o) return LBM_ERR_ARG;
-  std::memset(o, 0, sizeof(*o));
-  o->tau = 1.0;
-  o->bc_top_bottom = LBM_BC_FREESLIP;
-  o->storage = LBM_F32;
-  o->history_capacity = 1ll << 20;
-  o->kernel = LBM_KERNEL_AUTO;
-  o->ctas_per_sm = 0;  // the tuned default of the chosen shape
-  o->collision = LBM_COLLIDE_BGK;
-  o->s_e = o->s_eps = o->s_q = 1.1;
-  return LBM_OK;
-}
-
-int lbm_workspace_bytes(const lbm_opts *o, const uint8_t *mask, size_t *bytes) {
+int lattice_bytes(const lbm_opts *o, const uint8_t *mask, bool pair_tables, size_t *bytes) {
   int rc = check_opts(o);
   if (rc) return rc;
   if (!bytes) return LBM_ERR_ARG;
@@ -310,11 +296,11 @@ int lbm_workspace_bytes(const lbm_opts *o, const uint8_t *mask, size_t *bytes) {
   if (rc) return rc;
   int pitch, slot_cap, band_rows;
   size_t offs[kLayoutParts];
-  *bytes = layout(o, g, &pitch, offs, &slot_cap, &band_rows);
+  *bytes = layout(o, g, pair_tables, &pitch, offs, &slot_cap, &band_rows);
   return LBM_OK;
 }
 
-int lbm_create_ex(const lbm_opts *o, const uint8_t *mask, lbm_ctx **out) {
+int create_lattice(const lbm_opts *o, const uint8_t *mask, bool pair_tables, lbm_ctx **out) {
   if (!out) return LBM_ERR_ARG;
   *out = nullptr;
   int rc = check_opts(o);
@@ -332,7 +318,7 @@ int lbm_create_ex(const lbm_opts *o, const uint8_t *mask, lbm_ctx **out) {
   c->elem = elem_size(o->storage);
   c->ops = ops_for(o->storage);
   size_t offs[kLayoutParts];
-  c->ws_bytes = layout(o, c->geo, &c->pitch, offs, &c->slot_cap, &c->band_rows);
+  c->ws_bytes = layout(o, c->geo, pair_tables, &c->pitch, offs, &c->slot_cap, &c->band_rows);
   c->plane = (long long)c->ny * c->pitch;
   c->hist_cap = o->history_capacity > 0 ? o->history_capacity : (1ll << 20);
   auto fail = [&](int code) {
@@ -367,7 +353,7 @@ int lbm_create_ex(const lbm_opts *o, const uint8_t *mask, lbm_ctx **out) {
   c->staging_bytes = offs[7] - offs[6];
   c->wave_slots = (double2 *)(base + offs[7]);
   c->wave_rows = (unsigned *)(base + offs[8]);
-  c->pair_region = base + offs[9];
+  c->pair_region = offs[10] > offs[9] ? base + offs[9] : nullptr;
   if (o->stream) {
     c->stream = (cudaStream_t)o->stream;
   } else {
@@ -430,6 +416,30 @@ int lbm_create_ex(const lbm_opts *o, const uint8_t *mask, lbm_ctx **out) {
   *out = c;
   return LBM_OK;
 }
+
+}  // namespace gblbm
+
+extern "C" {
+
+int lbm_opts_default(lbm_opts *o) {
+  if (!o) return LBM_ERR_ARG;
+  std::memset(o, 0, sizeof(*o));
+  o->tau = 1.0;
+  o->bc_top_bottom = LBM_BC_FREESLIP;
+  o->storage = LBM_F32;
+  o->history_capacity = 1ll << 20;
+  o->kernel = LBM_KERNEL_AUTO;
+  o->ctas_per_sm = 0;  // the tuned default of the chosen shape
+  o->collision = LBM_COLLIDE_BGK;
+  o->s_e = o->s_eps = o->s_q = 1.1;
+  return LBM_OK;
+}
+
+int lbm_workspace_bytes(const lbm_opts *o, const uint8_t *mask, size_t *bytes) {
+  return lattice_bytes(o, mask, true, bytes);
+}
+
+int lbm_create_ex(const lbm_opts *o, const uint8_t *mask, lbm_ctx **out) { return create_lattice(o, mask, true, out); }
 
 int lbm_create(int nx, int ny, double tau, double U, const uint8_t *mask, int bc, lbm_ctx **out) {
   lbm_opts o;

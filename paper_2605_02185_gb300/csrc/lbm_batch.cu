@@ -75,7 +75,7 @@ int batch_sizes(int n, const lbm_case *cases, const lbm_opts *common, std::vecto
   for (int c = 0; c < n; ++c) {
     lbm_opts o = case_opts(*common, cases[c]);
     size_t b = 0;
-    const int rc = lbm_workspace_bytes(&o, cases[c].mask, &b);
+    const int rc = lattice_bytes(&o, cases[c].mask, false, &b);
     if (rc) return rc;
     (*sizes)[c] = align_up(b, kAlign);
     sum += (*sizes)[c];
@@ -256,7 +256,7 @@ int lbm_batch_create(int ncases, const lbm_case *cases, const lbm_opts *common, 
     o.workspace_bytes = sizes[c];
     off += sizes[c];
     lbm_ctx *ctx = nullptr;
-    rc = lbm_create_ex(&o, cases[c].mask, &ctx);
+    rc = create_lattice(&o, cases[c].mask, false, &ctx);
     if (rc) return fail(rc);
     b->cases.push_back(ctx);
   }

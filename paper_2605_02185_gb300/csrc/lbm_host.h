@@ -200,5 +200,9 @@ inline int default_batch_shape(int storage) { return storage == LBM_F64 ? 6 : 19
 inline int default_batch_ctas(int storage) { return storage == LBM_F64 ? 1 : 2; }
 inline int default_kernel(int storage) { return storage == LBM_F64 ? LBM_KERNEL_DIRECT : LBM_KERNEL_TMA; }
 
+// lbm_workspace_bytes and lbm_create_ex, with or without room for the two-step kernel's
+// tables: a batch has them once, for all its cases.
+int lattice_bytes(const lbm_opts *o, const uint8_t *mask, bool pair_tables, size_t *bytes);
+int create_lattice(const lbm_opts *o, const uint8_t *mask, bool pair_tables, lbm_ctx **out);
 
 }  // namespace gblbm
