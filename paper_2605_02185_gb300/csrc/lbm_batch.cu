@@ -116,10 +116,10 @@ int configure_batch(lbm_batch *b, int kernel, int shape, int ctas) {
   }
   const KernelOps *ops = b->cases[0]->ops;
   if (kernel != LBM_KERNEL_DIRECT) CK(ops->batch_prep(shape));
-  b->kernel = kernel;
-  b->shape = shape;
   const int rc = upload_desc(b);
   if (rc) return rc;
+  b->kernel = kernel;
+  b->shape = shape;
   b->ctas = kernel == LBM_KERNEL_DIRECT ? 0 : b->cases[0]->ctas_per_sm;
   b->grid = kernel == LBM_KERNEL_DIRECT ? (int)b->nitems : (int)std::min<long long>(b->nitems, (long long)b->sms * b->ctas);
   return LBM_OK;
