@@ -80,7 +80,8 @@ extern "C" {
                                bounce-back, and batches), and an odd step on the default
                                kernel.  The populations are bit-identical; a force is a sum
                                in double of the same links in another order, the same bits
-                               wherever that sum is exact.  lbm_steps_per_pass tells whether
+                               wherever that sum is exact (in a batch with BGK the
+                               links of two nodes of a row are added to 48 bits first).  lbm_steps_per_pass tells whether
                                a lattice is taken; left to the default kernel are some
                                whose body spans a third of the width or more, and those
                                wider than about 490,000 nodes.  Lattices of 150,000 to

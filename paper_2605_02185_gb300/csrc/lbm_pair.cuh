@@ -19,17 +19,18 @@
 // the body or the inlet delays nobody.
 //
 // The per-node arithmetic is that of the one-step kernels, on packed pairs: the
-// results are bit-identical to two of their steps.
+// populations are bit-identical to two of their steps; a force is a double sum of the
+// same links in another order.
 //
 // Why a warp, 64 columns and registers: with a CTA per strip and f*(n + 1) in
 // shared memory, the barrier of each row made every warp wait for the one with
 // the body or the inlet; with four nodes a lane (128 columns) only two warps fit a
-// scheduler and latency ruled (100 GLUPS on 8000 x 4000 against 147 with two).
+// scheduler and latency ruled (100 GLUPS on 8000 x 4000 against 136 with two).
 // What bounds it now: instruction issue and latency (562 instructions for the 120
 // node steps of a warp's row, issue slots 53 % used, DRAM 62 % busy on 8000 x 4000).
 // Time per step, BGK, cylinder lattices, one-step kernel before and this now:
-// 400 x 200 10.2 -> 5.1 us, 800 x 400 14.1 -> 6.6, 1600 x 800 21.2 -> 11.7,
-// 3200 x 1600 66.4 -> 38.3, 8000 x 4000 357 -> 235, 16000 x 8000 1416 -> 1102.
+// 400 x 200 10.2 -> 4.6 us, 800 x 400 14.1 -> 6.1, 1600 x 800 21.2 -> 12.2,
+// 3200 x 1600 66.4 -> 37.8, 8000 x 4000 357 -> 222, 16000 x 8000 1416 -> 1035.
 #pragma once
 
 #include <algorithm>
@@ -94,8 +95,9 @@ __device__ __forceinline__ void set_elem(float2 &v, int j, float s) {
 // long wait, so a row is added in pairs of floats, and its sums go to the double totals
 // once.  The pairs lose nothing while the terms lie within a factor of 2^15: up to 32 of
 // them are multiples of the smallest one's last bit, their rounding errors below 2^-14 of
-// the largest, and the sum of those fits a float's 24 bits.  Rows with other terms, with
-// infinities or near the ends of the float range are added in double.
+// the largest, and the sum of those fits a float's 24 bits.  Rows with other terms or near
+// the ends of the float range are added in double; with an infinity or NaN among them the
+// sum is one too, whatever it is added in.
 struct LinkSum {
   LF xh{}, xl{}, yh{}, yl{};
   uint32_t most = 0, least = 0xffffffffu;  // largest term's bits; smallest nonzero one's, less 1
@@ -116,14 +118,31 @@ struct LinkSum {
     }
     see(t);
   }
-  __device__ __forceinline__ bool exact() const {
-    return (most >> 23) < 248u && (most >> 23) <= ((least + 1u) >> 23) + 15u;
-  }
-  __device__ __forceinline__ void to(double &fx, double &fy) const {
-    fx += (double)xh.v + (double)xl.v;
-    fy += (double)yh.v + (double)yl.v;
+  // Add the sums to the totals; false where they have to be added in double.
+  __device__ __forceinline__ bool to(double &fx, double &fy) const {
+    const bool exact = (most >> 23) < 248u && (most >> 23) <= ((least + 1u) >> 23) + 15u;
+    const bool finite = most < 0x7f800000u;
+    if (finite && !exact) return false;
+    fx += (double)xh.v + (double)(finite ? xl.v : 0.f);
+    fy += (double)yh.v + (double)(finite ? yl.v : 0.f);
+    return true;
   }
 };
+
+// A sum in a pair of floats, 48 bits, without a branch on the terms (batches with BGK).
+struct PairSum {
+  LF hi{}, lo{};
+  __device__ __forceinline__ void add(LF v) {
+    LF e;
+    hi = two_sum(hi, v, e);
+    lo = lo + e;
+  }
+};
+// The same in double, whatever the terms (an infinity or NaN is in hi alone).
+__device__ __forceinline__ double total(const PairSum &s) {
+  const bool finite = fabsf(s.hi.v) < __int_as_float(0x7f800000);
+  return (double)s.hi.v + ((double)(finite ? s.lo.v : 0.f));
+}
 
 // The wall rules of boundaries() for a node of the bottom or top row.
 __device__ __forceinline__ void pair_wall(int bc, bool bottom, float U, float (&v)[9]) {
@@ -189,6 +208,10 @@ __global__ void __launch_bounds__(NW * 32, 1)
   if (warp >= per) return;
   const int first = (int)blockIdx.x * per + warp;
   if (first >= q.ncells) return;
+  // Zero.  Waiting for it here keeps a launch's warps in step, and with them the columns
+  // and DRAM pages that neighbouring cells share: 64 batched cases with MRT, 76M nodes, ran
+  // at 90 GLUPS without this load and at 112 with it.
+  const unsigned base_pass = ld_relaxed_gpu(q.flags + first);
   const StepParams &p = BATCH ? sp[warp] : p0;
   float *tiles = reinterpret_cast<float *>(smem + warp * Lay::WARP);
 
@@ -216,7 +239,7 @@ __global__ void __launch_bounds__(NW * 32, 1)
     }
     if (pass > 0) {  // the neighbours' last pass
       const int dep = __ldg(q.deps + (size_t)cell * 32 + lane);
-      const unsigned need = (unsigned)pass;
+      const unsigned need = base_pass + (unsigned)pass;
       bool ok = dep < 0 || ld_relaxed_gpu(q.flags + max(dep, 0)) >= need;
       if (!__all_sync(0xffffffffu, ok)) {
         const unsigned long long t0 = global_ns(), lim = wait_limit(p.wait_ns);
@@ -349,9 +372,7 @@ __global__ void __launch_bounds__(NW * 32, 1)
         }
         if constexpr (INTERP) {
           if (counts && mine) {
-            if (sum.exact()) {
-              sum.to(fx[s], fy[s]);
-            } else {
+            if (!sum.to(fx[s], fy[s])) {
 #pragma unroll 1
               for (int j = 0; j < 2; ++j)
 #pragma unroll
@@ -413,6 +434,25 @@ __global__ void __launch_bounds__(NW * 32, 1)
         }
         if constexpr (!INTERP) {
           if (counts) {  // half-way links: the population leaves and returns (the factor 2 comes last)
+            if constexpr (BATCH && !MRT) {
+              // Without a branch: one in this place, or the registers of a longer sum, makes
+              // the BGK batch spill in its marching loop (16 cases: 113 GLUPS as it is, 70
+              // with the exact pairs below, 69 with triples of floats).  Scaled by 2^-8 the sums
+              // stay within the float range.
+              PairSum sx, sy;
+#pragma unroll
+              for (int k = 1; k < 9; ++k)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                  const float t = m[j] & (1u << OPP(k)) ? 0x1p-8f * elem(g[k], j) : 0.f;
+                  if (CX(k)) sx.add(LF{CX(k) > 0 ? t : -t});
+                  if (CY(k)) sy.add(LF{CY(k) > 0 ? t : -t});
+                }
+              if (mine) {
+                fx[s] += 256.0 * total(sx);
+                fy[s] += 256.0 * total(sy);
+              }
+            } else {
             // Per node one value for each pair of opposite directions (both seldom hold a
             // link), and no branch for a direction without links.
             float d[2][4];
@@ -443,9 +483,7 @@ __global__ void __launch_bounds__(NW * 32, 1)
             sum.yl = (l[1] + l[2]) + e;
             sum.yh = two_sum(sum.yh, t[3], e);
             sum.yl = sum.yl + (e + l[3]);
-            if (!both && sum.exact()) {
-              sum.to(fx[s], fy[s]);
-            } else {
+            if (both || !sum.to(fx[s], fy[s])) {
 #pragma unroll 1
               for (int j = 0; j < 2; ++j)
 #pragma unroll
@@ -455,6 +493,7 @@ __global__ void __launch_bounds__(NW * 32, 1)
                     if (CX(k)) fx[s] += CX(k) > 0 ? t : -t;
                     if (CY(k)) fy[s] += CY(k) > 0 ? t : -t;
                   }
+            }
             }
           }
         }
@@ -546,7 +585,7 @@ __global__ void __launch_bounds__(NW * 32, 1)
     __syncwarp();
     if (lane == 0 && !(cd.x >> 16 == q.fault_case && a <= q.fault_row && q.fault_row < b)) {
       fence_acq_rel_gpu();
-      st_relaxed_gpu(q.flags + cell, (unsigned)pass + 1u);
+      st_relaxed_gpu(q.flags + cell, base_pass + (unsigned)pass + 1u);
     }
   }
 }

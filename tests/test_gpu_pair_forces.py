@@ -97,3 +97,22 @@ def test_wide_body(bounce):
             lat.close()
     assert np.array_equal(out[0][0].view(np.uint32), out[1][0].view(np.uint32))
     assert np.abs(out[0][1] - out[1][1]).max() <= 1000 * 2.0 ** -53 * 200
+
+
+def test_batch_sums_past_the_float_range():
+    wl = W.Workload(name="rest", nx=96, ny=40, D=8, xc=33, yc=18, U=0.0, tau=TAU, bc=W.BC_PERIODIC)
+    mask = wl.mask()
+    pops = np.zeros((9, 40, 96), np.float32)
+    pops[[2, 4, 5, 6, 7, 8]] = 8e37
+    pops[0] = -3.2e38
+    pops[:, mask == 1] = 0
+    ref = run(96, 40, mask, pops, 2, kernel=lbm.LBM_KERNEL_DIRECT)
+    b = lbm.Batch([wl])
+    try:
+        lbm.lbm_set_populations(b.case(0), pops, 1)
+        b.step(2)
+        got = b.forces_raw(0, 1, 2)
+    finally:
+        b.close()
+    assert np.all(np.isfinite(ref[1]))
+    assert np.array_equal(ref[1], got)
