@@ -31,8 +31,10 @@ constexpr double kCellCost = 3.0;
 // Nodes from which a launch runs one pass only.  Within a launch the cells drift
 // apart, and on a large lattice the columns and DRAM pages that neighbouring
 // windows share are then fetched twice; the launch between passes lines them up
-// again.  3200 x 1600: 38.8 us a step with 32 passes a launch, 43.4 with one;
-// 8000 x 4000: 259 and 235; 16000 x 8000: 1224 and 1117.
+// again.  us a step with 32 passes a launch and with one: 3200 x 1600 41 and 45,
+// 4400 x 2200 (9.7M nodes) 75.3 and 77.1, 4800 x 2400 92.9 and 91.3, 5600 x 2800 (15.7M)
+// 126 and 121, 6400 x 3200 172 and 155, 8000 x 4000 259 and 235: the two meet near 10M
+// nodes, and between there and this line up to 4 % is left.
 constexpr long long kPairManyNodes = 16ll << 20;
 
 // Windows of a row: the last one yields column nx - 2 (and column nx - 1, its

@@ -17,10 +17,11 @@
 // mma.sync kernel for 8 channels, whose K steps of 16 are half zeros), so the
 // sums are the same bits.  Every wait is bounded as in nn_tc.cu.
 //
-// 4 samples, us before (conv_tc_kernel; 8 channels: mma.sync) and now: 800 x 1600,
-// forward 32 -> 32 457 and 165, 8 -> 32 594 and 113, 32 -> 8 457 and 130, 96 -> 32
-// 700 and 655; gradient 32 -> 32 450 and 215, 32 -> 96 862 and 720; 400 x 800,
-// 32 -> 64 162 and 90, 64 -> 64 154 and 104, its gradient 158 and 160.  What bounds
+// 4 samples, us before (conv_tc_kernel; 8 channels: mma.sync) and now, both without a
+// mask: 800 x 1600, forward 32 -> 32 457 and 169, 8 -> 32 594 and 122, 32 -> 8 457 and 126,
+// 96 -> 32 700 and 655; gradient 32 -> 32 450 and 157, 32 -> 96 862 and 416; 400 x 800,
+// 32 -> 64 162 and 104, 64 -> 64 154 and 105, its gradient 158 and 102.  Small images are
+// left to conv_tc_kernel (nn_rows_rule.h).  What bounds
 // it: 32 -> 32 DRAM at half its rate, with the latency of the read-back and the
 // row copies of two resident CTAs; 96 -> 32 the MMAs, each reading 4 KB of A for 32
 // columns.
